@@ -259,9 +259,10 @@ typedef struct {
                                            (default 3) */
     int32_t nonuniform_kernel_f32;      /* FP32 rows with their own mesh: 0 = the
                                            per-order kernels (shared-memory-free without
-                                           a residual, tiled with one; the default),
-                                           1 = the warp-segment kernel (one launch for
-                                           every order, shift and residual together) */
+                                           a residual, tiled with one), 1 = the
+                                           warp-segment kernel (one launch for every
+                                           order, shift and residual together; what a
+                                           new plan takes) */
 } ram_tuning;
 
 ram_status ram_plan_get_tuning(ram_plan plan, ram_tuning *out);

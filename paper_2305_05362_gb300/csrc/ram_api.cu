@@ -60,6 +60,7 @@ StepArgs base_args(const Plan *p, const void *q_in, void *q_out)
     a.dx64 = p->dx64;
     a.buckets = p->buckets;
     a.density = p->density;
+    a.x32 = p->x32;
     a.wait_limit = p->wait_limit;
     return a;
 }

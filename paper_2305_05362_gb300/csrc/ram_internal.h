@@ -30,8 +30,8 @@ struct RowInfo {
     int32_t order;        // 2, 3, 4
     int32_t uniform;      // 1: equal widths, O(1) edge index
     int32_t bucket_bits;  // log2 of the row's bucket count
-    int32_t qshift;       // FP32 warp-segment kernel: window-relative fixed-point
-                          // positions are kept as 32-bit values in units of 2^qshift
+    int32_t qshift;       // FP32 warp-segment kernel: positions are kept as 32-bit values
+                          // (modulo 2^32) in units of 2^qshift
     int32_t density;      // index of the row's mesh-density function, -1: none
     double period;        // L
     double cells_per_length;  // N / L
@@ -67,15 +67,16 @@ struct Tile {
 constexpr int kGenHalo = 2 * RAM_MAX_NSUB;
 constexpr int kGenHR = 2;
 
-// FP32 rows with their own mesh: the warp-segment kernel (ram_nseg.cu).  A lane
-// forms the reconstructions of kNsegV consecutive window cells; a segment has
-// at most kNseg output cells; a CTA of kNsegWarps warps takes a tile of up to
-// kNsegWarps * kNsegPerWarp segments.
-constexpr int kNsegV = 4;
-constexpr int kNseg = 96;
+// FP32 rows with their own mesh: the warp-segment kernel (ram_nseg.cu).  A warp
+// stages a window of kNsegWin source cells and takes segments of at most
+// kNsegMost output cells, residual halo included; a CTA of kNsegWarps warps takes
+// up to kNsegItems of them.
+constexpr int kNsegWin = 160;
 constexpr int kNsegHR = 2;          // reconstruction halo, cells per side
-constexpr int kNsegWarps = 8;
-constexpr int kNsegPerWarp = 4;
+constexpr int kNsegMost = kNsegWin - 8;
+constexpr int kNsegWarps = 4;
+constexpr int kNsegItems = 64;
+constexpr int kNsegCtas = 6;        // resident CTAs per SM
 // shortest row it takes (a segment and its residual halo span less than a period)
 constexpr int kNsegMinCells = 2 * kGenHalo + 2;
 
@@ -106,6 +107,7 @@ struct StepArgs {
     const double *dx64;     // widths, FP64
     const int32_t *buckets; // per-row bucket table: cell holding each bucket start
     const Density *density; // mesh-density functions of rows that have one
+    const uint32_t *x32;    // xfix >> qshift, the low 32 bits (warp-segment rows)
     uint32_t wait_limit = kWaitLimit;  // tries of every bounded mbarrier wait
     int32_t row_phase = 0;  // no parameter kernel ran: the row kernels advance the phase
 };
@@ -127,6 +129,7 @@ template <typename T> struct RowParams {
 // the plan
 struct Plan {
     int device = 0;
+    int32_t sm_count = 152;
     int32_t n_rows = 0;
     int64_t n_cells = 0;
     uint32_t flags = 0;
@@ -168,7 +171,9 @@ struct Plan {
     void *a4_scratch = nullptr;
     std::vector<Tile> tiles_nseg_h;
     int32_t nseg_rows = 0;
-    int32_t nu_kernel = 0;         // FP32 rows with their own mesh: 1 = warp-segment kernel
+    int32_t nu_kernel = 1;         // FP32 rows with their own mesh: 1 = warp-segment kernel
+    std::vector<int32_t> nseg_cells_h;  // per row: most cells of a segment with its halo, 0:
+                                        // the row does not take the warp-segment kernel
     // uniform rows taken by the persistent whole-row kernel, per dtype and order, and
     // the tiles of the remaining uniform rows
     std::vector<int32_t> rows_fit_h[2][5];
@@ -205,6 +210,7 @@ struct Plan {
     void *row_par = nullptr;        // RowParams<double> per row (FP32 launches use the first
                                     // half of each slot as RowParams<float>)
     uint64_t *xfix = nullptr;
+    uint32_t *x32 = nullptr;
     float *dx32 = nullptr;
     double *dx64 = nullptr;
     int32_t *buckets = nullptr;
@@ -239,10 +245,6 @@ cudaError_t launch_uniform(const Plan &p, ram_dtype dt, const StepArgs &a, cudaS
 cudaError_t launch_general(const Plan &p, ram_dtype dt, const StepArgs &a, cudaStream_t s);
 // FP32 rows with their own mesh, warp-segment kernel (ram_nseg.cu)
 cudaError_t launch_nseg(const Plan &p, const StepArgs &a, cudaStream_t s);
-size_t nseg_smem_bytes(bool resid);
-// largest source window (cells) a warp of it stages; rows above it take the tiled
-// kernels
-int nseg_window_cap();
 cudaError_t launch_row_mass(const Plan &p, ram_dtype dt, const void *q, double *out,
                             cudaStream_t s);
 cudaError_t launch_adjoint(const Plan &p, ram_dtype dt, const StepArgs &a, const void *g_out,

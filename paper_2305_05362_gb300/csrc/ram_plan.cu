@@ -101,6 +101,8 @@ void free_device(Plan &p)
     cudaFree(p.rows);
     free_lists(p);
     cudaFree(p.xfix);
+    cudaFree(p.x32);
+    p.x32 = nullptr;
     cudaFree(p.dx32);
     cudaFree(p.dx64);
     cudaFree(p.buckets);
@@ -129,55 +131,80 @@ std::vector<double> doubled_widths(const double *x, int n)
     return w2;
 }
 
-// The longest physical extent of `span` consecutive cells (cyclic), and the most
-// source cells an interval that long can touch, over every placement: for every
-// start st, cells st..e-1 fit strictly inside it; it also touches cell e and the
-// cell st-1 it may start in.
-int most_cells_touched(const std::vector<double> &w2, int n, int span)
+// What the FP32 warp-segment kernel takes of a row: the most cells of a segment
+// with its residual halo (0: the row is left to the tiled kernels), and the units
+// 2^qs of its 32-bit positions.  x: nodes; w: widths.
+//
+// The positions of a window and of the edges over it span less than 2^32 units; rows
+// not much longer than that take half the period's units, so that two turns fit.
+// Every cell keeps at least 2^20 units, and one output cell lies over fewer source
+// cells than a window holds (both from sums over whole rows of the widths).
+//
+// A segment whose source cells do not fit one window costs another window, so the
+// length is the one with the least expected cost per output cell, windows over
+// output cells, on 64 sampled placements: 144 cells on widths of [1/2, 2] x mean
+// (against 128 for placements that all fit: 61 and 68 us on the 512-row batch).
+int nseg_cells(const double *x, const double *w, int n, int &qs)
 {
-    double len_max = 0.0, acc = 0.0;
-    for (int k = 0; k < span; ++k) acc += w2[k % (2 * n)];
-    len_max = acc;
-    for (int st = 1; st < n; ++st) {
-        acc += w2[(st + span - 1) % (2 * n)] - w2[st - 1];
-        len_max = std::max(len_max, acc);
+    qs = 0;
+    if (n < kNsegMinCells) return 0;
+    const int room = kNsegWin - 2 * kNsegHR;
+    const double L = x[n] - x[0];
+    double w_min = w[0], w_max = w[0], reach = 2.0 * L;
+    for (int i = 1; i < n; ++i) {
+        w_min = std::min(w_min, w[i]);
+        w_max = std::max(w_max, w[i]);
+    }
+    const int span = kNsegWin + 2;
+    if (n > span) {
+        double len = 0.0;
+        for (int st = 0; st < n; ++st)
+            len = std::max(len, st + span <= n ? x[st + span] - x[st]
+                                               : x[st + span - n] - x[st] + L);
+        reach = len + w_max;
+    }
+    const double two64 = 18446744073709551616.0;
+    if (reach > 0.999 * L)
+        qs = 33;
+    else
+        qs = std::max(0, (int)std::ceil(std::log2(reach / L * two64 * 1.000001)) - 32);
+    if (std::ldexp(w_min / L * two64, -qs) < 1048576.0) return 0;
+    if (w_max > w_min * (room - 8)) {
+        // the most cells an interval as long as the widest cell can touch
+        int e = 0;
+        double len = 0.0;  // of cells st .. e - 1 (cyclic)
+        for (int st = 0; st < n; ++st) {
+            while (e < st + n && len + w[e % n] < w_max) len += w[e++ % n];
+            if (e - st + 2 > room - 8) return 0;
+            if (e > st)
+                len -= w[st];
+            else
+                e = st + 1;
+        }
     }
     int best = 0;
-    acc = 0.0;
-    int e = 0;
-    for (int st = 0; st < n; ++st) {
-        if (e < st) {
-            e = st;
-            acc = 0.0;
+    double cost = 1e300;
+    for (int ne = kNsegMost; ne >= 64; ne -= 8) {
+        const int c = std::min(ne, n - 1);
+        double windows = 0.0;
+        for (int k = 0; k < 64; ++k) {
+            const int i = (int)((2654435761ull * (2 * k + 1)) % (uint64_t)n);
+            const int j = (int)((40503ull * 65537ull * (2 * k + 1) + n / 3) % (uint64_t)n);
+            double len = (i + c <= n ? x[i + c] - x[i] : x[i + c - n] - x[i] + L) + x[j];
+            int turn = 0;
+            if (len > x[n]) {
+                len -= L;
+                turn = n;
+            }
+            const int e = (int)(std::upper_bound(x, x + n + 1, len) - x) + turn;
+            windows += std::max(1, (e - j + room - 2) / (room - 1));
         }
-        while (e < st + n && acc + w2[e] < len_max) acc += w2[e++];
-        best = std::max(best, e - st + 2);
-        if (e > st) acc -= w2[st];
+        if (windows / (c - 4) < cost) {
+            cost = windows / (c - 4);
+            best = c;
+        }
     }
-    return std::min(best, n + 1);
-}
-
-// Units (a power of two of fixed-point length, 2^qs) in which the FP32
-// warp-segment kernel keeps window-relative positions as 32-bit values: every
-// window of up to `wb` cells must span less than 2^31 units, and every cell at
-// least 2^21 (so that in-cell offsets keep about 21 significant bits); -1 when
-// the row's widths vary too much for both.
-int position_shift(const std::vector<double> &w2, int n, int wb, double L)
-{
-    double acc = 0.0, len_max = 0.0, w_min = w2[0];
-    for (int k = 0; k < wb; ++k) acc += w2[k % (2 * n)];
-    len_max = acc;
-    for (int st = 1; st < n; ++st) {
-        acc += w2[(st + wb - 1) % (2 * n)] - w2[st - 1];
-        len_max = std::max(len_max, acc);
-    }
-    for (int i = 0; i < n; ++i) w_min = std::min(w_min, w2[i]);
-    const double two64 = 18446744073709551616.0;
-    const double lfix = std::min(len_max / L, 1.0) * two64;
-    int qs = std::max(0, (int)std::floor(std::log2(lfix)) - 30);
-    if (std::ldexp(lfix, -qs) >= 2147483648.0) ++qs;
-    if (std::ldexp(w_min / L * two64, -qs) < 2097152.0) return -1;
-    return qs;
+    return best;
 }
 
 // The general kernels' per-order launch shapes of a tile list: whole-row tiles
@@ -284,39 +311,16 @@ ram_status build_tiles(Plan &p)
         // the adjoint's tiles: plain runs of at most adj_nu_tcap cells
         for (int a = 0; a < n; a += p.adj_nu_tcap)
             p.tiles_adj_nu_h[ri.order].push_back(Tile{r, a, std::min(p.adj_nu_tcap, n - a), 0});
-        // FP32: the warp-segment kernel, with segments short enough that a segment
-        // and its largest residual halo span less than a period, and a source
-        // window that fits its shared-memory region
-        bool nseg = false;
-        p.rows_h[r].qshift = 0;
-        if (n >= kNsegMinCells) {
-            // the longest segment whose source window, residual halo included, fits
-            // the warp's window; preferably one whose window without a residual
-            // fits half of it (one pass of the reconstruction)
-            const int cap = nseg_window_cap();
-            const int seg_max = std::min(kNseg, n - 1 - 2 * kGenHalo);
-            int seg = 0, wb = 0;
-            for (int pass = 0; pass < 2 && seg == 0; ++pass) {
-                for (int sg = seg_max; sg >= 1; sg -= (sg > 8 ? 8 : sg)) {
-                    const int w1 = most_cells_touched(w2, n, sg + 2 * kGenHalo) + 2 * kNsegHR + 1;
-                    const int w0 = most_cells_touched(w2, n, sg) + 2 * kNsegHR + 1;
-                    if (w1 <= cap && (pass == 1 || w0 <= cap / 2)) {
-                        seg = sg;
-                        wb = w1;
-                        break;
-                    }
-                    if (sg < kNseg / 3) break;
-                }
-            }
-            int qs = -1;
-            if (seg > 0) qs = position_shift(w2, n, wb, x[n] - x[0]);
-            if (qs >= 0) {
-                nseg = true;
-                ++p.nseg_rows;
-                p.rows_h[r].qshift = qs;
-                const int per_tile = seg * kNsegWarps * kNsegPerWarp;
-                for (int a = 0; a < n; a += per_tile)
-                    p.tiles_nseg_h.push_back(Tile{r, a, std::min(per_tile, n - a), seg});
+        // FP32: the warp-segment kernel's items, near-equal segments that leave room
+        // for the halo of one van Leer sub-step (wider halos are cut in the kernel)
+        const bool nseg = p.nseg_cells_h[r] > 0;
+        if (nseg) {
+            ++p.nseg_rows;
+            const int most = p.nseg_cells_h[r];
+            const int64_t ns = (n + std::max(1, most - 4) - 1) / std::max(1, most - 4);
+            for (int64_t k = 0; k < ns; ++k) {
+                const int a = (int)(n * k / ns), b = (int)(n * (k + 1) / ns);
+                p.tiles_nseg_h.push_back(Tile{r, a, b - a, most});
             }
         }
         std::vector<Tile> &g32 = p.tiles_general32_h[ri.order];
@@ -376,10 +380,6 @@ ram_status build_tiles(Plan &p)
         if (upload(&p.tiles_adj_nu[o], p.tiles_adj_nu_h[o].data(), p.tiles_adj_nu_h[o].size()) !=
             cudaSuccess)
             return RAM_ERR_NOMEM;
-    // the rows' position units (qshift) live in the device row table
-    if (p.rows && cudaMemcpy(p.rows, p.rows_h.data(), sizeof(RowInfo) * p.rows_h.size(),
-                             cudaMemcpyHostToDevice) != cudaSuccess)
-        return RAM_ERR_CUDA;
     for (int o = 2; o <= 4; ++o) {
         // the general kernel runs whole-row tiles (window 0) and windowed tiles as
         // two launches, each with the shared memory its own largest tile needs
@@ -457,6 +457,8 @@ extern "C" ram_status ram_plan_mesh(const ram_mesh_desc *desc, int device, ram_p
         return RAM_ERR_NOMEM;
     }
     p->device = device;
+    if (cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+        p->sm_count = 152;
     p->n_rows = nr;
     p->n_cells = ro[nr];
     p->flags = desc->flags;
@@ -476,17 +478,20 @@ extern "C" ram_status ram_plan_mesh(const ram_mesh_desc *desc, int device, ram_p
     std::vector<float> dx32;
     std::vector<double> dx64;
     std::vector<int32_t> buckets;
+    std::vector<uint32_t> x32;
     // order 4 with the limiter on (the scaled quartic) runs on the general kernels:
     // the uniform-row kernels fold a row's partial integrals into constants
     bool limited4 = false;
     for (int r = 0; r < nr; ++r)
         limited4 |= p->limiter && (desc->order ? desc->order[r] : desc->default_order) == 4;
     p->rows_h.resize(nr);
+    p->nseg_cells_h.assign(nr, 0);
     for (int r = 0; r < nr && st == RAM_OK; ++r) {
         const int n = (int)(ro[r + 1] - ro[r]);
         const double *x = shared ? p->nodes_h.data() : p->nodes_h.data() + ro[r] + r;
         RowInfo &ri = p->rows_h[r];
         ri.density = -1;
+        ri.qshift = 0;
         ri.cell_off = ro[r];
         ri.n = n;
         ri.order = desc->order ? desc->order[r] : desc->default_order;
@@ -499,6 +504,8 @@ extern "C" ram_status ram_plan_mesh(const ram_mesh_desc *desc, int device, ram_p
             ri.mesh_off = p->rows_h[0].mesh_off;
             ri.bucket_off = p->rows_h[0].bucket_off;
             ri.bucket_bits = p->rows_h[0].bucket_bits;
+            ri.qshift = p->rows_h[0].qshift;
+            p->nseg_cells_h[r] = p->nseg_cells_h[0];
             continue;
         }
         st = check_nodes(x, n);
@@ -529,6 +536,13 @@ extern "C" ram_status ram_plan_mesh(const ram_mesh_desc *desc, int device, ram_p
             dx64[base + i] = x[i + 1] - x[i];
             dx32[base + i] = (float)dx64[base + i];
         }
+        x32.resize(base + n);
+        if (!ri.uniform) {
+            int qs = 0;
+            p->nseg_cells_h[r] = nseg_cells(x, dx64.data() + base, n, qs);
+            ri.qshift = qs;
+            for (int i = 0; i < n; ++i) x32[base + i] = (uint32_t)(xfix[base + i] >> qs);
+        }
         int bits = 1;
         while ((1LL << bits) < 2LL * n && bits < 40) ++bits;
         ri.bucket_bits = bits;
@@ -555,6 +569,7 @@ extern "C" ram_status ram_plan_mesh(const ram_mesh_desc *desc, int device, ram_p
     if (st == RAM_OK) {
         if (upload(&p->rows, p->rows_h.data(), p->rows_h.size()) != cudaSuccess ||
             upload(&p->xfix, xfix.data(), xfix.size()) != cudaSuccess ||
+            upload(&p->x32, x32.data(), x32.size()) != cudaSuccess ||
             upload(&p->dx32, dx32.data(), dx32.size()) != cudaSuccess ||
             upload(&p->dx64, dx64.data(), dx64.size()) != cudaSuccess ||
             upload(&p->buckets, buckets.data(), buckets.size()) != cudaSuccess ||
