@@ -75,7 +75,7 @@ constexpr int kNsegWin = 160;
 constexpr int kNsegHR = 2;          // reconstruction halo, cells per side
 constexpr int kNsegMost = kNsegWin - 8;
 constexpr int kNsegWarps = 4;
-constexpr int kNsegItems = 64;
+constexpr int kNsegItems = 48;
 constexpr int kNsegCtas = 6;        // resident CTAs per SM
 // shortest row it takes (a segment and its residual halo span less than a period)
 constexpr int kNsegMinCells = 2 * kGenHalo + 2;

@@ -85,7 +85,8 @@ constexpr int kOffR = kOffM + kWin + 4;      // node positions relative to the w
 constexpr int kOffP = kOffR + 256 + 4;       // the segment's new values
 constexpr int kOffV = kOffP + kWin + 4;      // dv at the segment's nodes (residual)
 constexpr int kWords = kOffV;
-constexpr int kWordsResid = kOffV + kWin + 4;
+constexpr int kOffH = kOffV + kWin + 4;      // widths of the segment's cells (residual)
+constexpr int kWordsResid = kOffH + kWin + 4;
 static_assert(kOffC % 4 == 0 && kWords % 4 == 0 && kWordsResid % 4 == 0, "16-byte aligned");
 
 // Coefficients of the in-cell cumulative G(d) = d (c0 + d (c1 + d (c2 + d c3))) of
@@ -204,15 +205,15 @@ struct Item {
     int32_t order, qs;
     int32_t p;                 // source cell of the first edge (halo included)
     int32_t nsub;
-    float cf;                  // mean widths swept per unit dv in a sub-step
-    float scale;               // position units -> mean widths
+    float cf;                  // sub-step length
+    float scale;               // position units -> the widths' units, about mean widths
 };
 
 struct SegCtx {
     const uint32_t *X32;
     const float *qin;
     float *qout;
-    const float *dvp;
+    const float *dvp, *dx;
     int N, H, nsub, lane, hi;  // hi: first window node past the cells an edge may lie in
     bool vl;
     float scale, cf;
@@ -299,7 +300,9 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
     for (int i = 0; i <= kV; ++i) xo[i] = sE[b + i];
     const uint32_t x_first = sE[0], x_last = sE[ne];
     if (RESID) {
-        // dv of the segment's nodes: needed after the remap
+        // dv of the segment's nodes and its cells' widths: needed after the remap (the
+        // rounded nodes would do for the remap alone, whose masses they share; against
+        // dv dt they leave the narrow cells of a graded row 2^-20)
         const int a0 = i0 - g.H < 0 ? i0 - g.H + N : i0 - g.H;
         const uint32_t d = smem_u32(sV);
 #pragma unroll 1
@@ -307,6 +310,7 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
             int c = a0 + k;
             c = c >= N ? c - N : c;  // ne < N
             cp_async4(d + 4u * k, g.dvp + c);
+            cp_async4(d + 4u * (kOffH - kOffV) + 4u * k, g.dx + c);
         }
     }
     cp_async_commit();
@@ -475,7 +479,7 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
         for (int i = 0; i < kV; ++i) {
             cur[i] = sP[b + i];
             c[i] = sV[b + i] * g.cf;  // signed length swept by node i in a sub-step
-            h[i] = (float)(xo[i + 1] - xo[i]) * g.scale;
+            h[i] = sV[kOffH - kOffV + b + i];
             rh[i] = rcp_approx(h[i]);
         }
         const float hm = __shfl_up_sync(full, h[kV - 1], 1), hp = __shfl_down_sync(full, h[0], 1);
@@ -556,14 +560,17 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
     pdl_wait();
     pdl_trigger();
     if (tid < n_it) {
+        const uint64_t *X = a.xfix + row.mesh_off;
+        int ns = RESID && a.nsub ? a.nsub[t.row] : (RESID ? 1 : 0);
+        if (RESID) ns = ns < 1 ? 1 : (ns > RAM_MAX_NSUB ? RAM_MAX_NSUB : ns);
+        int e = t.start - ns * R;
+        e = e < 0 ? e + row.n : e;
+        const uint64_t xe = X[e];  // in flight while the shift is formed
         // the row's first item advances the phase when no parameter kernel ran
         RowParams<float> P;
         shift_params<float>(a, row, t.row, a.row_phase != 0 && t.start == 0, P);
         const uint64_t S = P.sfix;
         const int qs = row.qshift;
-        const uint64_t *X = a.xfix + row.mesh_off;
-        int e = t.start - P.nsub * R;
-        e = e < 0 ? e + row.n : e;
         Item it;
         it.cell_off = row.cell_off;
         it.mesh_off = row.mesh_off;
@@ -575,11 +582,12 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
         it.order = row.order;
         it.qs = qs;
         it.p = locate_cell(X, row.n, a.buckets + row.bucket_off, row.bucket_bits, a.density,
-                           row.density, X[e] - S);
+                           row.density, xe - S);
         it.S = S;
         it.nsub = P.nsub;
-        it.cf = P.cf * (float)row.cells_per_length;
-        it.scale = (float)row.n * __int_as_float((127 + qs - 64) << 23);
+        it.cf = P.cf;
+        // a power of two, so that widths and offsets round once; a mean cell is in [1, 2)
+        it.scale = __int_as_float((127 + qs - 64 + 32 - __clz(row.n)) << 23);
         s_item[tid] = it;
     }
     __syncthreads();
@@ -642,6 +650,7 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
         g.qin = static_cast<const float *>(a.q_in) + it.cell_off;
         g.qout = static_cast<float *>(a.q_out) + it.cell_off;
         g.dvp = RESID ? static_cast<const float *>(a.dv) + it.cell_off : nullptr;
+        g.dx = a.dx32 + it.mesh_off;
         g.N = it.n;
         g.nsub = it.nsub;
         g.H = RESID ? it.nsub * R : 0;
