@@ -13,11 +13,16 @@
 // the forward sub-step states are recomputed from the step input.  The upwind
 // side at c_j = 0 is the left cell.
 //
-// Launch: blockIdx.y = 0 computes g_in for a tile of source cells, blockIdx.y = 1
-// adds dL/d dv for the tile's interfaces (each interface in exactly one tile, so
-// there are no atomics).
+// Two kernels.  k_adj_seg (rows of at least 512 cells on 16-byte boundaries) gives
+// each warp a run of output cells, V a lane, in registers: one pass over g, dv and
+// the step input forms both gradients, neighbours by shuffles, and FP32 rows form
+// their shift themselves (no parameter kernel).  k_adj_uniform takes the other rows:
+// blockIdx.y = 0 computes g_in for a tile of source cells, blockIdx.y = 1 adds dL/d
+// dv for the tile's interfaces (each interface in exactly one tile, so there are no
+// atomics).
 #include <cuda_runtime.h>
 
+#include <cstdint>
 #include <vector>
 
 #include "ram_device.cuh"
@@ -48,6 +53,216 @@ __device__ __forceinline__ void alpha_coeffs(const RowParams<T> &P, T al[5])
         al[4] = -b * P.c[1];
     } else {
         for (int s = 0; s < 5; ++s) al[s] = P.c[s];
+    }
+}
+
+// beta_u (u = -2..3) from the left partial's coefficients
+template <typename T, int ORDER>
+__device__ __forceinline__ void beta_coeffs(const RowParams<T> &P, T beta[6])
+{
+    T al[5];
+    alpha_coeffs<T, ORDER>(P, al);
+#pragma unroll
+    for (int u = -2; u <= 3; ++u)
+        beta[u + 2] = (u == 0 ? T(1) : T(0)) - (u <= 2 ? al[u <= 2 ? u + 2 : 0] : T(0)) +
+                      (u >= -1 ? al[u >= -1 ? u + 1 : 0] : T(0));
+}
+
+constexpr int kSegWarps = 4;
+
+// Cells per lane of the warp-segment kernel.
+template <typename T> constexpr int kSegV = sizeof(T) == 4 ? 8 : 4;
+
+// Halo cells at each end of a warp's 32 V cells, whole 16-byte vectors: the sub-steps
+// spoil nsub cells at each end, the gather takes 2 on the left and 3 on the right.
+template <typename T> __host__ __device__ constexpr int seg_halo(int nsub)
+{
+    return (nsub + 3 + 16 / (int)sizeof(T) - 1) / (16 / (int)sizeof(T)) * (16 / (int)sizeof(T));
+}
+
+__device__ __forceinline__ int wrap_twice(int c, int N)  // c within (-2N, 2N)
+{
+    if (c < 0) c += N;
+    if (c < 0) c += N;
+    if (c >= N) c -= N;
+    if (c >= N) c -= N;
+    return c;
+}
+
+template <typename T> struct Vec16;
+template <> struct Vec16<float> {
+    using V = float4;
+};
+template <> struct Vec16<double> {
+    using V = double2;
+};
+
+// M values (whole vectors) from row cells first, first + 1, ... (cyclic; first and N
+// whole vectors, first in [0, N)), the lane's.
+template <typename T, int M>
+__device__ __forceinline__ void load_cells(const T *row, int first, int N, T (&out)[M])
+{
+    using V = typename Vec16<T>::V;
+    constexpr int VEC = 16 / sizeof(T);
+#pragma unroll
+    for (int c = 0; c < M / VEC; ++c) {
+        const int i = first + c * VEC;
+        const V v = *reinterpret_cast<const V *>(row + (i >= N ? i - N : i));
+        const T *e = reinterpret_cast<const T *>(&v);
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) out[c * VEC + k] = e[k];
+    }
+}
+
+// One warp per segment of output cells [out0, out0 + stride) of a row, its 32 V cells
+// from out0 - H on; lane l holds V consecutive ones.  In one pass: the states of the
+// donor sub-steps from the step input (state k from state 0 again for each k: one or
+// two sub-steps in earnest), the sub-steps' transpose in reverse with dL/d dv, and
+// the shift's transpose, g_in[m - K] = sum_u beta_u g'[m + 1 - u].  The shift by K
+// leaves g_in unaligned, so it passes through shared memory to be stored a lane a
+// word.
+//
+// Bound by latency and the launch at 512 x 2048 cells, where a step's 24 bytes a cell
+// stay in L2; the tile passes of k_adj_uniform, with the parameter kernel before
+// them, took 30.6 us there, this 7.3 (FP32, PPM, one or two sub-steps).  A segment a
+// warp, so that few rows still fill the SMs.
+template <typename T, int ORDER>
+__global__ void __launch_bounds__(kSegWarps * 32)
+    k_adj_seg(StepArgs a, const int32_t *row_ids, const RowParams<T> *pars, const T *g_out,
+              T *g_in, T *g_dv)
+{
+    constexpr int V = kSegV<T>, VEC = 16 / sizeof(T);
+    using Vec = typename Vec16<T>::V;
+    __shared__ __align__(16) T stage[kSegWarps][32 * V];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int seg = blockIdx.y * kSegWarps + warp;
+    const int r = row_ids[blockIdx.x];
+    const RowInfo row = a.rows[r];
+    pdl_wait();
+    pdl_trigger();
+    RowParams<T> P;
+    if constexpr (sizeof(T) == 4)
+        shift_params_two_float(a, row, r, seg == 0 && lane == 0, P);
+    else
+        P = pars[r];
+    const int N = row.n, nsub = P.nsub;
+    const int H = seg_halo<T>(nsub);
+    const int stride = 32 * V - 2 * H;
+    const int out0 = seg * stride;
+    if (out0 >= N) return;
+    const unsigned full = 0xffffffffu;
+    const int m0 = out0 - H + lane * V;  // the lane's first cell (may wrap)
+    const int mc = wrap_twice(m0, N);
+
+    T g[V];
+    load_cells<T, V>(g_out + row.cell_off, mc, N, g);
+    T beta[6];
+    beta_coeffs<T, ORDER>(P, beta);
+    if (nsub > 0) {
+        T cp[V + 1], cm[V];  // upwind parts of the faces' Courant numbers (face i: left node)
+        {
+            T c[V];
+            load_cells<T, V>(static_cast<const T *>(a.dv) + row.cell_off, mc, N, c);
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                c[i] *= P.cf;
+                cp[i] = fmax(c[i], T(0));
+                cm[i] = fmin(c[i], T(0));
+            }
+            cp[V] = __shfl_down_sync(full, cp[0], 1);
+        }
+        T acc[V], q0[V];
+#pragma unroll
+        for (int i = 0; i < V; ++i) acc[i] = T(0);
+        if (g_dv != nullptr) {
+            // the shifted field: source cells p - 2 .. p + V + 2, p = m0 - K - 1, from a
+            // vector boundary
+            const int off = ((-P.K - 1) % VEC + VEC) % VEC;
+            T w[V + 3 * VEC];
+            load_cells<T, V + 3 * VEC>(static_cast<const T *>(a.q_in) + row.cell_off,
+                                       wrap_twice(wrap_twice(m0, N) - P.K - 1 - off - VEC, N), N, w);
+#pragma unroll
+            for (int o = 0; o < VEC; ++o)
+                if (o == off) {
+#pragma unroll
+                    for (int i = 0; i < V; ++i) {
+                        // w[o + VEC + i + u] holds cell p + i + u
+                        T v = T(0);
+#pragma unroll
+                        for (int u = -2; u <= 3; ++u) v += beta[u + 2] * w[o + VEC + i + u];
+                        q0[i] = P.whole ? w[o + VEC + i + 1] : v;
+                    }
+                }
+        }
+        for (int k = nsub - 1; k >= 0; --k) {
+            // transposed flux differences h_i = g_i - g_{i-1}
+            T h[V + 1];
+            h[0] = g[0] - __shfl_up_sync(full, g[V - 1], 1);
+#pragma unroll
+            for (int i = 1; i < V; ++i) h[i] = g[i] - g[i - 1];
+            h[V] = __shfl_down_sync(full, h[0], 1);
+            if (g_dv != nullptr) {
+                T q[V];
+#pragma unroll
+                for (int i = 0; i < V; ++i) q[i] = q0[i];
+                for (int s = 0; s < k; ++s) {
+                    const T zl = __shfl_up_sync(full, q[V - 1], 1);
+                    T F[V + 1];
+#pragma unroll
+                    for (int i = 0; i < V; ++i) F[i] = fma(cp[i], i ? q[i - 1] : zl, cm[i] * q[i]);
+                    F[V] = __shfl_down_sync(full, F[0], 1);
+#pragma unroll
+                    for (int i = 0; i < V; ++i) q[i] -= F[i + 1] - F[i];
+                }
+                const T zl = __shfl_up_sync(full, q[V - 1], 1);
+#pragma unroll
+                for (int i = 0; i < V; ++i) {
+                    // the upwind cell, the left one at c = 0
+                    const T qu = cm[i] < T(0) ? q[i] : (i ? q[i - 1] : zl);
+                    acc[i] = fma(qu, h[i], acc[i]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < V; ++i) g[i] = fma(cp[i + 1], h[i + 1], fma(cm[i], h[i], g[i]));
+        }
+        if (g_dv != nullptr) {
+            T *gd = g_dv + row.cell_off;
+#pragma unroll
+            for (int c = 0; c < V / VEC; ++c) {
+                const int li = lane * V + c * VEC, m = m0 + c * VEC;
+                if (li >= H && li < H + stride && m < N) {
+                    Vec v = *reinterpret_cast<const Vec *>(gd + m);
+                    T *e = reinterpret_cast<T *>(&v);
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) e[k] = fma(P.cf, acc[c * VEC + k], e[k]);
+                    *reinterpret_cast<Vec *>(gd + m) = v;
+                }
+            }
+        }
+    }
+
+    // ---- the shift's transpose: local cell i gives g_in[m0 + i - K] ----
+    T e[V + 5];  // g' at local cells -2 .. V + 2
+    e[0] = __shfl_up_sync(full, g[V - 2], 1);
+    e[1] = __shfl_up_sync(full, g[V - 1], 1);
+#pragma unroll
+    for (int i = 0; i < V; ++i) e[i + 2] = g[i];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) e[V + 2 + i] = __shfl_down_sync(full, g[i], 1);
+    T *st = stage[warp];
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+        T v = T(0);
+#pragma unroll
+        for (int u = -2; u <= 3; ++u) v += beta[u + 2] * e[i + 3 - u];
+        st[lane * V + i] = P.whole ? g[i] : v;
+    }
+    __syncwarp();
+    T *gi = g_in + row.cell_off;
+    const int cnt = min(stride, N - out0);
+    for (int k = lane; k < cnt; k += 32) {
+        const int j = out0 + k - P.K;
+        gi[j < 0 ? j + N : j] = st[H + k];
     }
 }
 
@@ -201,14 +416,13 @@ __global__ void __launch_bounds__(256)
 }
 
 template <typename T, int ORDER>
-cudaError_t launch_adj_t(const Plan &p, const StepArgs &a, const void *g_out, void *g_in,
-                         void *g_dv, cudaStream_t s)
+cudaError_t launch_adj_tiles(const Plan &p, const StepArgs &a, const Tile *tiles,
+                             const std::vector<Tile> &th, const void *g_out, void *g_in,
+                             void *g_dv, cudaStream_t s)
 {
-    const std::vector<Tile> &th = p.tiles_uniform_h[ORDER];
     if (th.empty()) return cudaSuccess;
     int cap = 0;
     for (const Tile &t : th) cap = cap > t.count ? cap : t.count;
-    if (cap > 256 * 8) return cudaErrorNotSupported;
     const int wcap = cap + 2 * kMaxSub + 16;
     const size_t smem = sizeof(T) * ((size_t)3 * wcap + 1 + (size_t)kMaxSub * wcap);
     if (smem > 227 * 1024) return cudaErrorNotSupported;
@@ -222,11 +436,48 @@ cudaError_t launch_adj_t(const Plan &p, const StepArgs &a, const void *g_out, vo
         configured[dev] = smem;
     }
     StepArgs b = a;
-    b.tiles = p.tiles_uniform[ORDER];
+    b.tiles = tiles;
     b.n_tiles = (int)th.size();
     return launch_pdl(k_adj_uniform<T, ORDER>, dim3((int)th.size(), 2), 256, smem, s, b,
                       static_cast<const RowParams<T> *>(p.row_par), static_cast<const T *>(g_out),
                       static_cast<T *>(g_in), static_cast<T *>(g_dv), cap);
+}
+
+// The warp-segment kernel reads and writes 16-byte vectors of every array but g_in.
+bool seg_aligned(const StepArgs &a, const void *g_out, const void *g_dv)
+{
+    for (const void *ptr : {a.q_in, a.dv, g_out, g_dv})
+        if ((uintptr_t)ptr % 16) return false;
+    return true;
+}
+
+template <typename T, int ORDER>
+cudaError_t launch_adj_t(const Plan &p, const StepArgs &a, const void *g_out, void *g_in,
+                         void *g_dv, bool vec, cudaStream_t s)
+{
+    constexpr int d = sizeof(T) == 4 ? 0 : 1;
+    for (const Tile &t : p.tiles_uniform_h[ORDER])
+        if (t.count > 256 * 8) return cudaErrorNotSupported;  // tiles k_adj_uniform does not take
+    if (!vec)
+        return launch_adj_tiles<T, ORDER>(p, a, p.tiles_uniform[ORDER], p.tiles_uniform_h[ORDER],
+                                          g_out, g_in, g_dv, s);
+    const std::vector<int32_t> &rows = p.rows_seg_h[d][ORDER];
+    if (!rows.empty()) {
+        int n = 0;
+        for (int32_t r : rows) n = n > p.rows_h[r].n ? n : p.rows_h[r].n;
+        // segments of the longest row at the widest halo; the warps past a row's end leave
+        const int stride = 32 * kSegV<T> - 2 * seg_halo<T>(a.dv ? RAM_MAX_NSUB : 0);
+        const int y = ((n + stride - 1) / stride + kSegWarps - 1) / kSegWarps;
+        cudaError_t e = launch_pdl(k_adj_seg<T, ORDER>, dim3((unsigned)rows.size(), y),
+                                   dim3(kSegWarps * 32), 0, s, a,
+                                   static_cast<const int32_t *>(p.rows_seg[d][ORDER]),
+                                   static_cast<const RowParams<T> *>(p.row_par),
+                                   static_cast<const T *>(g_out), static_cast<T *>(g_in),
+                                   static_cast<T *>(g_dv));
+        if (e != cudaSuccess) return e;
+    }
+    return launch_adj_tiles<T, ORDER>(p, a, p.tiles_rest_seg[d][ORDER], p.tiles_rest_seg_h[d][ORDER],
+                                      g_out, g_in, g_dv, s);
 }
 
 }  // namespace
@@ -239,16 +490,20 @@ cudaError_t launch_adjoint(const Plan &p, ram_dtype dt, const StepArgs &a, const
     if (nonuni && a.dv != nullptr && p.adj_scratch == nullptr) return cudaErrorNotSupported;
     // a limited plan: every row on the gather adjoint, linearised at the step input
     if (p.adj_all) return launch_adjoint_nu(p, dt, a, g_out, g_in, g_dv, s);
-    cudaError_t e = launch_params(p, dt, a, s);
+    const bool vec = seg_aligned(a, g_out, g_dv);
+    // FP32 warp-segment rows form their own shift
+    bool params = dt != RAM_F32 || nonuni || !vec;
+    for (int o = 2; o <= 4; ++o) params |= !p.tiles_rest_seg_h[0][o].empty();
+    cudaError_t e = params ? launch_params(p, dt, a, s) : cudaSuccess;
     if (e != cudaSuccess) return e;
     if (dt == RAM_F32) {
-        if ((e = launch_adj_t<float, 2>(p, a, g_out, g_in, g_dv, s)) != cudaSuccess) return e;
-        if ((e = launch_adj_t<float, 3>(p, a, g_out, g_in, g_dv, s)) != cudaSuccess) return e;
-        if ((e = launch_adj_t<float, 4>(p, a, g_out, g_in, g_dv, s)) != cudaSuccess) return e;
+        if ((e = launch_adj_t<float, 2>(p, a, g_out, g_in, g_dv, vec, s)) != cudaSuccess) return e;
+        if ((e = launch_adj_t<float, 3>(p, a, g_out, g_in, g_dv, vec, s)) != cudaSuccess) return e;
+        if ((e = launch_adj_t<float, 4>(p, a, g_out, g_in, g_dv, vec, s)) != cudaSuccess) return e;
     } else {
-        if ((e = launch_adj_t<double, 2>(p, a, g_out, g_in, g_dv, s)) != cudaSuccess) return e;
-        if ((e = launch_adj_t<double, 3>(p, a, g_out, g_in, g_dv, s)) != cudaSuccess) return e;
-        if ((e = launch_adj_t<double, 4>(p, a, g_out, g_in, g_dv, s)) != cudaSuccess) return e;
+        if ((e = launch_adj_t<double, 2>(p, a, g_out, g_in, g_dv, vec, s)) != cudaSuccess) return e;
+        if ((e = launch_adj_t<double, 3>(p, a, g_out, g_in, g_dv, vec, s)) != cudaSuccess) return e;
+        if ((e = launch_adj_t<double, 4>(p, a, g_out, g_in, g_dv, vec, s)) != cudaSuccess) return e;
     }
     return nonuni ? launch_adjoint_nu(p, dt, a, g_out, g_in, g_dv, s) : cudaSuccess;
 }

@@ -1,0 +1,58 @@
+"""The warp-segment transpose of uniform rows where its ranges end: rows of the
+shortest length it takes, of one segment more or less, whole-cell and seam shifts,
+one to eight sub-steps (the widest halo), arrays off the 16-byte boundary (the tiled
+kernel), against the FP64 oracle at the suite's bars (relative L1 <= 1e-12 FP64,
+1e-5 FP32)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+from paper_2305_05362_gb300 import ram, workloads as wl
+from gpu_common import TOL
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+SHIFTS = [0.0, 3.0, 511.0, 0.4, 7.3, -1.25, 300.62]  # cells, one row each
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("n", [508, 512, 516, 744, 748, 1000, 2052])
+@pytest.mark.parametrize("order,nsub", [(2, 1), (3, 2), (4, 8), (3, 5), (3, 0)])
+def test_matches_oracle(dtype, n, order, nsub):
+    x = wl.uniform_nodes(n, 0.25, 2.0)
+    rows = len(SHIFTS)
+    plan = ram.Plan(np.arange(rows + 1) * n, x, order=order, limiter=False, shared_mesh=True)
+    rng = np.random.default_rng(n + nsub)
+    dt = 0.5
+    dx = 2.0 / n
+
+    def put(a, off=0):
+        buf = torch.empty(a.size + off, dtype=dtype, device=DEV)[off:]
+        return buf.copy_(torch.tensor(a, device=DEV))
+
+    q, g = rng.standard_normal((2, rows * n))
+    dv = (rng.random(rows * n) - 0.5) * 1.6 * max(nsub, 1) * dx / dt
+    g0 = rng.standard_normal(rows * n)
+    v0 = torch.tensor(np.array(SHIFTS) * dx / dt, device=DEV)
+    ns = torch.full((rows,), max(nsub, 1), dtype=torch.int32, device=DEV)
+    results = []
+    for off in (0, 1):
+        qd, gd, dvd, gdv = put(q, off), put(g), put(dv), put(g0)
+        gin = torch.empty_like(gd)
+        ram.step_adjoint(plan, qd, gd, gin, v0, dt, dv=dvd if nsub else None,
+                         g_dv=gdv if nsub else None, nsub=ns)
+        results.append((gin.double().cpu().numpy(), gdv.double().cpu().numpy()))
+    tol = TOL["float64" if dtype == torch.float64 else "float32"]
+    qr, gr, dvr, g0r = (t.double().cpu().numpy() for t in (put(q), put(g), put(dv), put(g0)))
+    for r in range(rows):
+        sl = slice(r * n, (r + 1) * n)
+        ri, rd = oracle.step_adjoint(x, qr[sl], gr[sl], oracle.shift_from_velocity(float(v0[r]), dt),
+                                     order, dvr[sl] if nsub else None, dt, max(nsub, 1))
+        for gin, gdv in results:
+            assert np.abs(gin[sl] - ri).sum() <= tol * np.abs(ri).sum(), r
+            if nsub:
+                ref = g0r[sl] + rd  # added into what was there
+                assert np.abs(gdv[sl] - ref).sum() <= tol * (np.abs(g0r[sl]) + np.abs(rd)).sum(), r
+    assert plan.check_errors() == 0
