@@ -169,6 +169,26 @@ ram_status ram_step_adjoint(ram_plan plan, ram_dtype dtype, const void *q_in,
                             const void *dv_iface, void *g_dv, const int32_t *nsub,
                             void *stream);
 
+/* k >= 1 calls of ram_step in a row, each on the result of the one before, with the
+ * same arguments (no phase).  states NULL: the last writes q_out, the others alternate
+ * between q_out and scratch (n_cells values; needed when k > 1).  Otherwise every state
+ * is kept, state i (0 .. k-1) at states + i pitch values (pitch >= n_cells), and q_out
+ * and scratch are not used.  The buffers must not overlap each other or q_in
+ * (RAM_ERR_ARG).  Stops at the first call that does not return RAM_OK, with its status. */
+ram_status ram_steps(ram_plan plan, ram_dtype dtype, const void *q_in, void *q_out, void *scratch,
+                     void *states, int64_t pitch, int32_t k, const double *v0, double dt,
+                     const void *dv_iface, ram_scheme scheme, const int32_t *nsub, void *stream);
+
+/* The transposes of the k >= 1 steps that ram_steps takes from q_in with the donor
+ * residual, last to first: k calls of ram_step_adjoint, step i's input q_in (i = 0) or
+ * state i - 1 (states and pitch as ram_steps keeps them; k - 1 states are read).  The
+ * cotangent goes from g_out to g_in through scratch (n_cells values; needed when
+ * k > 1); g_dv as in ram_step_adjoint, added to by every step. */
+ram_status ram_steps_adjoint(ram_plan plan, ram_dtype dtype, const void *q_in, const void *states,
+                             int64_t pitch, int32_t k, const void *g_out, void *g_in,
+                             void *scratch, const double *v0, double dt, const void *dv_iface,
+                             void *g_dv, const int32_t *nsub, void *stream);
+
 /* The radial sweep of a polar disk, for dimensional splitting in two dimensions
  * (Sec. 3.5: RAM along the azimuth, a standard upwind step along the radius).  The
  * plan must have RAM_SHARED_MESH (RAM_ERR_UNSUPPORTED otherwise): its rows are the

@@ -25,31 +25,25 @@ class RamSegment(torch.autograd.Function):
         ctx.plan, ctx.v0, ctx.dt, ctx.nsub, ctx.k = plan, v0, dt, nsub, k
         q = q.contiguous()
         ctx.save_for_backward(q, dv)
-        cur = q
-        for _ in range(k):
-            nxt = torch.empty_like(cur)
-            ram.step(plan, cur, nxt, v0, dt, dv=dv, scheme=ram.DONOR, nsub=nsub)
-            cur = nxt
-        return cur
+        if k < 1:
+            return q
+        out = torch.empty_like(q)
+        ram.steps(plan, q, out, k, v0, dt, dv=dv, scheme=ram.DONOR, nsub=nsub)
+        return out
 
     @staticmethod
     def backward(ctx, g):
         q, dv = ctx.saved_tensors
         plan, v0, dt, nsub, k = ctx.plan, ctx.v0, ctx.dt, ctx.nsub, ctx.k
-        states = [q]
-        for _ in range(k - 1):
-            nxt = torch.empty_like(q)
-            ram.step(plan, states[-1], nxt, v0, dt, dv=dv, scheme=ram.DONOR, nsub=nsub)
-            states.append(nxt)
         g = g.contiguous()
         g_dv = None
         if dv is not None and ctx.needs_input_grad[1]:
             g_dv = torch.zeros_like(dv)
-        for i in reversed(range(k)):
-            gin = torch.empty_like(g)
-            ram.step_adjoint(plan, states[i], g, gin, v0, dt, dv=dv, g_dv=g_dv, nsub=nsub)
-            g = gin
-        return g, g_dv, None, None, None, None, None
+        if k < 1:
+            return g, g_dv, None, None, None, None, None
+        g_in = torch.empty_like(g)
+        ram.steps_adjoint(plan, q, g, g_in, k, v0, dt, dv=dv, g_dv=g_dv, nsub=nsub)
+        return g_in, g_dv, None, None, None, None, None
 
 
 def rollout(plan, q0, v0, dt: float, steps: int, dv=None, nsub=None,

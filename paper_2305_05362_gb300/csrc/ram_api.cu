@@ -28,12 +28,14 @@ struct DeviceGuard {
 
 size_t dtype_size(ram_dtype d) { return d == RAM_F64 ? 8 : 4; }
 
-bool overlaps(const void *a, const void *b, size_t bytes)
+bool overlaps2(const void *a, size_t a_bytes, const void *b, size_t b_bytes)
 {
     const char *x = static_cast<const char *>(a);
     const char *y = static_cast<const char *>(b);
-    return x < y + bytes && y < x + bytes;
+    return x < y + b_bytes && y < x + a_bytes;
 }
+
+bool overlaps(const void *a, const void *b, size_t bytes) { return overlaps2(a, bytes, b, bytes); }
 
 ram_status check_common(const Plan *p, ram_dtype dt, const void *q_in, const void *q_out)
 {
@@ -215,6 +217,66 @@ extern "C" ram_status ram_step_adjoint(ram_plan plan, ram_dtype dtype, const voi
                                    static_cast<cudaStream_t>(stream));
     if (e == cudaErrorNotSupported) return RAM_ERR_UNSUPPORTED;
     return e == cudaSuccess ? RAM_OK : RAM_ERR_CUDA;
+}
+
+extern "C" ram_status ram_steps(ram_plan plan, ram_dtype dtype, const void *q_in, void *q_out,
+                                void *scratch, void *states, int64_t pitch, int32_t k,
+                                const double *v0, double dt, const void *dv_iface,
+                                ram_scheme scheme, const int32_t *nsub, void *stream)
+{
+    const Plan *p = reinterpret_cast<const Plan *>(plan);
+    if (!p || k < 1 || (dtype != RAM_F32 && dtype != RAM_F64)) return RAM_ERR_ARG;
+    const size_t es = dtype_size(dtype), bytes = (size_t)p->n_cells * es;
+    if (states) {
+        if (pitch < p->n_cells || !q_in ||
+            overlaps2(q_in, bytes, states, ((size_t)(k - 1) * pitch) * es + bytes))
+            return RAM_ERR_ARG;
+    } else if (k > 1 && (!scratch || !q_in || !q_out || overlaps(q_in, q_out, bytes) ||
+                         overlaps(q_in, scratch, bytes) || overlaps(q_out, scratch, bytes))) {
+        return RAM_ERR_ARG;
+    }
+    const void *in = q_in;
+    for (int32_t i = 0; i < k; ++i) {
+        // the last one lands in q_out
+        void *out = states ? static_cast<char *>(states) + (size_t)i * pitch * es
+                           : ((k - 1 - i) % 2 ? scratch : q_out);
+        const ram_status st = ram_step(plan, dtype, in, out, nullptr, v0, dt, dv_iface, scheme,
+                                       nsub, stream);
+        if (st != RAM_OK) return st;
+        in = out;
+    }
+    return RAM_OK;
+}
+
+extern "C" ram_status ram_steps_adjoint(ram_plan plan, ram_dtype dtype, const void *q_in,
+                                        const void *states, int64_t pitch, int32_t k,
+                                        const void *g_out, void *g_in, void *scratch,
+                                        const double *v0, double dt, const void *dv_iface,
+                                        void *g_dv, const int32_t *nsub, void *stream)
+{
+    const Plan *p = reinterpret_cast<const Plan *>(plan);
+    if (!p || k < 1 || (dtype != RAM_F32 && dtype != RAM_F64)) return RAM_ERR_ARG;
+    const size_t es = dtype_size(dtype), bytes = (size_t)p->n_cells * es;
+    if (k > 1) {
+        if (!states || pitch < p->n_cells || !q_in || !g_out || !g_in || !scratch)
+            return RAM_ERR_ARG;
+        const size_t kept = (size_t)(k - 2) * pitch * es + bytes;
+        for (const void *w : {static_cast<const void *>(g_in), static_cast<const void *>(scratch)})
+            if (overlaps(w, g_out, bytes) || overlaps(w, q_in, bytes) ||
+                overlaps2(w, bytes, states, kept))
+                return RAM_ERR_ARG;
+        if (overlaps(g_in, scratch, bytes)) return RAM_ERR_ARG;
+    }
+    const void *g = g_out;
+    for (int32_t i = k - 1; i >= 0; --i) {
+        const void *q = i ? static_cast<const char *>(states) + (size_t)(i - 1) * pitch * es : q_in;
+        void *out = i % 2 ? scratch : g_in;  // step 0 lands in g_in
+        const ram_status st = ram_step_adjoint(plan, dtype, q, g, out, v0, dt, dv_iface, g_dv, nsub,
+                                               stream);
+        if (st != RAM_OK) return st;
+        g = out;
+    }
+    return RAM_OK;
 }
 
 extern "C" ram_status ram_row_mass(ram_plan plan, ram_dtype dtype, const void *q,

@@ -29,7 +29,7 @@ A4 = 8
 MAX_NSUB = 8
 
 EXPORTS = ["ram_plan_mesh", "ram_plan_destroy", "ram_shift", "ram_residual_upwind",
-           "ram_step", "ram_step_adjoint", "ram_row_mass", "ram_plan_check_errors",
+           "ram_step", "ram_step_adjoint", "ram_steps", "ram_steps_adjoint", "ram_row_mass", "ram_plan_check_errors",
            "ram_plan_query", "ram_plan_set_tiling", "ram_plan_set_wait_limit",
            "ram_plan_get_tuning", "ram_plan_set_tuning", "ram_plan_autotune", "ram_step_uniform_noalloc",
            "ram_radial_upwind", "ram_plan_set_density",
@@ -101,6 +101,10 @@ def load(path: Optional[str] = None):
     lib.ram_residual_upwind.argtypes = [vp, i32, vp, vp, vp, f64, i32, vp, vp]
     lib.ram_step.argtypes = [vp, i32, vp, vp, vp, vp, f64, vp, i32, vp, vp]
     lib.ram_step_adjoint.argtypes = [vp, i32, vp, vp, vp, vp, f64, vp, vp, vp, vp]
+    i64 = ctypes.c_int64
+    lib.ram_steps.argtypes = [vp, i32, vp, vp, vp, vp, i64, i32, vp, f64, vp, i32, vp, vp]
+    lib.ram_steps_adjoint.argtypes = [vp, i32, vp, vp, i64, i32, vp, vp, vp, vp, f64, vp, vp, vp,
+                                      vp]
     lib.ram_row_mass.argtypes = [vp, i32, vp, vp, vp]
     lib.ram_plan_check_errors.argtypes = [vp]
     lib.ram_plan_query.argtypes = [vp, ctypes.POINTER(PlanInfo)]
@@ -185,8 +189,66 @@ def _check_step_args(plan: "Plan", q_in, q_out, per_row=(), dv=None, nsub=None,
 def _stream(device: int, stream=None) -> int:
     import torch
     if stream is None:
-        stream = torch.cuda.current_stream(device)
+        return torch._C._cuda_getCurrentRawStream(device)
     return stream.cuda_stream
+
+
+def _fits(t, numel: int, dtype, device: int) -> bool:
+    """What _need and _ptr refuse, in one expression for the calls whose arguments are
+    as they should be (a step on a small plan takes the GPU 3 us, and naming each
+    argument's checks took the host 3.6): get_device is -1 for a CPU tensor."""
+    return (t.numel() == numel and t.dtype is dtype and t.get_device() == device
+            and t.is_contiguous())
+
+
+def _step_pointers(plan: "Plan", cells, rows, dv=None, nsub=None):
+    """Device pointers of the packed arrays `cells` ((name, tensor, optional), the first
+    one gives the dtype), the FP64 per-row arrays `rows`, dv and nsub, or None if any
+    of them is not what the plan takes (the caller then finds out which)."""
+    import torch
+    n, nr, dev = plan.n_cells, plan.n_rows, plan.device
+    dtype = cells[0][1].dtype
+    if dtype is not torch.float32 and dtype is not torch.float64:
+        return None
+    out = []
+    for _, t, optional in cells:
+        if t is None and optional:
+            out.append(None)
+        elif t is not None and _fits(t, n, dtype, dev):
+            out.append(t.data_ptr())
+        else:
+            return None
+    for _, t, optional in rows:
+        if t is None and optional:
+            out.append(None)
+        elif t is not None and _fits(t, nr, torch.float64, dev):
+            out.append(t.data_ptr())
+        else:
+            return None
+    if dv is None:
+        out.append(None)
+    elif _fits(dv, n, dtype, dev):
+        out.append(dv.data_ptr())
+    else:
+        return None
+    if nsub is None:
+        out.append(None)
+    elif _fits(nsub, nr, torch.int32, dev):
+        out.append(nsub.data_ptr())
+    else:
+        return None
+    return out
+
+
+def _pointers(plan: "Plan", cells, rows, dv=None, nsub=None):
+    """_step_pointers, or the ValueError / TypeError that says what does not fit."""
+    out = _step_pointers(plan, cells, rows, dv, nsub)
+    if out is None:
+        _check_step_args(plan, cells[0][1], cells[1][1], per_row=rows, dv=dv, nsub=nsub,
+                         extra_cells=cells[2:])
+        out = [_ptr(t) for _, t, _ in cells] + [_ptr(t) for _, t, _ in rows]
+        out += [_ptr(dv), _ptr(nsub)]
+    return out
 
 
 class Plan:
@@ -292,10 +354,10 @@ class Plan:
 
 def shift(plan: Plan, q_in, q_out, shift_per_row, stream=None):
     """ram_shift: remap every row by +shift[r]."""
-    _check_step_args(plan, q_in, q_out, per_row=[("shift", shift_per_row, False)])
-    _check(plan._lib.ram_shift(plan.handle, _dtype_code(q_in), _ptr(q_in), _ptr(q_out),
-                               _ptr(shift_per_row), _stream(plan.device, stream)),
-           "ram_shift")
+    qi, qo, sh, _, _ = _pointers(plan, (("q_in", q_in, False), ("q_out", q_out, False)),
+                                 (("shift", shift_per_row, False),))
+    _check(plan._lib.ram_shift(plan.handle, _dtype_code(q_in), qi, qo, sh,
+                               _stream(plan.device, stream)), "ram_shift")
 
 
 def residual_upwind(plan: Plan, q_in, q_out, dv, dt: float, scheme: int = VANLEER,
@@ -312,24 +374,63 @@ def residual_upwind(plan: Plan, q_in, q_out, dv, dt: float, scheme: int = VANLEE
 def step(plan: Plan, q_in, q_out, v0, dt: float, dv=None, scheme: int = VANLEER,
          nsub=None, phase=None, stream=None):
     """ram_step: shift by v0*dt then the residual step (dv=None: no residual)."""
-    _check_step_args(plan, q_in, q_out, per_row=[("v0", v0, False), ("phase", phase, True)],
-                     dv=dv, nsub=nsub)
-    _check(plan._lib.ram_step(plan.handle, _dtype_code(q_in), _ptr(q_in), _ptr(q_out),
-                              _ptr(phase), _ptr(v0), float(dt), _ptr(dv), int(scheme),
-                              _ptr(nsub), _stream(plan.device, stream)),
-           "ram_step")
+    qi, qo, v, ph, d, ns = _pointers(plan, (("q_in", q_in, False), ("q_out", q_out, False)),
+                                     (("v0", v0, False), ("phase", phase, True)), dv, nsub)
+    _check(plan._lib.ram_step(plan.handle, _dtype_code(q_in), qi, qo, ph, v, float(dt), d,
+                              int(scheme), ns, _stream(plan.device, stream)), "ram_step")
 
 
 def step_adjoint(plan: Plan, q_in, g_out, g_in, v0, dt: float, dv=None, g_dv=None,
                  nsub=None, stream=None):
     """ram_step_adjoint: g_in = J^T g_out of the linear step; adds into g_dv."""
-    _check_step_args(plan, g_out, g_in, per_row=[("v0", v0, False)], dv=dv, nsub=nsub,
-                     extra_cells=[("q_in", q_in, False), ("g_dv", g_dv, True)])
-    _check(plan._lib.ram_step_adjoint(plan.handle, _dtype_code(g_out), _ptr(q_in),
-                                      _ptr(g_out), _ptr(g_in), _ptr(v0), float(dt),
-                                      _ptr(dv), _ptr(g_dv), _ptr(nsub),
-                                      _stream(plan.device, stream)),
+    go, gi, qi, gd, v, d, ns = _pointers(
+        plan, (("g_out", g_out, False), ("g_in", g_in, False), ("q_in", q_in, False),
+               ("g_dv", g_dv, True)), (("v0", v0, False),), dv, nsub)
+    _check(plan._lib.ram_step_adjoint(plan.handle, _dtype_code(g_out), qi, go, gi, v, float(dt), d,
+                                      gd, ns, _stream(plan.device, stream)),
            "ram_step_adjoint")
+
+
+def _state_pitch(n_cells: int) -> int:
+    """Values from one kept state to the next: every state on a 256-byte boundary."""
+    return (n_cells + 63) // 64 * 64
+
+
+def steps(plan: Plan, q_in, q_out, k: int, v0, dt: float, dv=None, scheme: int = VANLEER,
+          nsub=None):
+    """ram_steps: k steps in a row from q_in, the last state into q_out, on the current
+    stream (which the scratch field belongs to)."""
+    import torch
+    k = int(k)
+    scratch = torch.empty_like(q_out) if k > 1 else None
+    qi, qo, sc, v, d, ns = _pointers(
+        plan, (("q_in", q_in, False), ("q_out", q_out, False), ("scratch", scratch, True)),
+        (("v0", v0, False),), dv, nsub)
+    _check(plan._lib.ram_steps(plan.handle, _dtype_code(q_in), qi, qo, sc, None, 0, k, v,
+                               float(dt), d, int(scheme), ns, _stream(plan.device)), "ram_steps")
+
+
+def steps_adjoint(plan: Plan, q_in, g_out, g_in, k: int, v0, dt: float, dv=None, g_dv=None,
+                  nsub=None):
+    """The transpose of `steps` (donor residual) from the same q_in: the states are taken
+    again (ram_steps) and walked back through (ram_steps_adjoint), on the current stream
+    (which the states belong to)."""
+    import torch
+    k = int(k)
+    n, pitch = plan.n_cells, _state_pitch(plan.n_cells)
+    scratch = torch.empty_like(g_in) if k > 1 else None
+    go, gi, qi, gd, sc, v, d, ns = _pointers(
+        plan, (("g_out", g_out, False), ("g_in", g_in, False), ("q_in", q_in, False),
+               ("g_dv", g_dv, True), ("scratch", scratch, True)), (("v0", v0, False),), dv, nsub)
+    states, code, s = None, _dtype_code(g_out), _stream(plan.device)
+    if k > 1:
+        states = torch.empty((k - 2) * pitch + n, dtype=q_in.dtype, device=q_in.device)
+        _check(plan._lib.ram_steps(plan.handle, code, qi, None, None, states.data_ptr(), pitch,
+                                   k - 1, v, float(dt), d, DONOR, ns, s), "ram_steps")
+    _check(plan._lib.ram_steps_adjoint(plan.handle, code, qi,
+                                       None if states is None else states.data_ptr(), pitch, k,
+                                       go, gi, sc, v, float(dt), d, gd, ns, s),
+           "ram_steps_adjoint")
 
 
 def autotune(plan: Plan, q_in, q_out, v0, dt: float, dv=None, scheme: int = VANLEER,

@@ -56,3 +56,34 @@ def test_matches_oracle(dtype, n, order, nsub):
                 ref = g0r[sl] + rd  # added into what was there
                 assert np.abs(gdv[sl] - ref).sum() <= tol * (np.abs(g0r[sl]) + np.abs(rd)).sum(), r
     assert plan.check_errors() == 0
+
+
+@pytest.mark.parametrize("n", [512, 515])
+@pytest.mark.parametrize("k", [1, 2, 3, 6])
+def test_steps_in_a_row_equal_single_calls(n, k):
+    """ram.steps and ram.steps_adjoint give what k single calls give, bit for bit (also
+    with an odd number of cells, where the kept states are padded)."""
+    plan = ram.Plan([0, n, 2 * n], wl.uniform_nodes(n), order=3, limiter=False, shared_mesh=True)
+    gen = torch.Generator(device=DEV).manual_seed(n + k)
+    q, g, dv = torch.randn(3, 2 * n, generator=gen, device=DEV).unbind(0)
+    dv = dv * (0.1 / n)
+    v0 = torch.tensor([0.013, -0.4], dtype=torch.float64, device=DEV)
+    out, g_in, g_dv = torch.empty_like(q), torch.empty_like(q), torch.ones_like(q)
+    ram.steps(plan, q, out, k, v0, 1.0, dv=dv, scheme=ram.DONOR)
+    ram.steps_adjoint(plan, q, g, g_in, k, v0, 1.0, dv=dv, g_dv=g_dv)
+    states, gd = [q.contiguous()], torch.ones_like(q)
+    for _ in range(k):
+        nxt = torch.empty_like(states[-1])
+        ram.step(plan, states[-1], nxt, v0, 1.0, dv=dv, scheme=ram.DONOR)
+        states.append(nxt)
+    assert torch.equal(out, states[-1])
+    for i in reversed(range(k)):
+        gi = torch.empty_like(q)
+        ram.step_adjoint(plan, states[i], g, gi, v0, 1.0, dv=dv, g_dv=gd)
+        g = gi
+    # (a misaligned field takes the tiled kernel: the same numbers to rounding)
+    close = dict(rtol=0, atol=0) if n % 4 == 0 else dict(rtol=1e-5, atol=1e-5)
+    torch.testing.assert_close(g_in, g, **close)
+    torch.testing.assert_close(g_dv, gd, **close)
+    with pytest.raises(ram.RamError):
+        ram.steps(plan, q, q, k, v0, 1.0, dv=dv)
