@@ -22,6 +22,7 @@
 // atomics).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <vector>
 
@@ -97,72 +98,54 @@ template <> struct Vec16<double> {
     using V = double2;
 };
 
-// M values (whole vectors) from row cells first, first + 1, ... (cyclic; first and N
-// whole vectors, first in [0, N)), the lane's.
-template <typename T, int M>
-__device__ __forceinline__ void load_cells(const T *row, int first, int N, T (&out)[M])
+// M values (whole vectors) from the lane's cells first, first + 1, ... (cyclic), first =
+// wfirst + lane V; wfirst is the warp's, in [0, N), whole vectors like N.
+template <typename T, int M, int V>
+__device__ __forceinline__ void load_cells(const T *row, int wfirst, int lane, int N, T (&out)[M])
 {
-    using V = typename Vec16<T>::V;
+    using Vec = typename Vec16<T>::V;
     constexpr int VEC = 16 / sizeof(T);
+    Vec v[M / VEC];
+    if (wfirst + 31 * V + M <= N) {
+        const T *src = row + wfirst + lane * V;
+#pragma unroll
+        for (int c = 0; c < M / VEC; ++c) v[c] = *reinterpret_cast<const Vec *>(src + c * VEC);
+    } else {
+#pragma unroll
+        for (int c = 0; c < M / VEC; ++c) {
+            const int i = wfirst + lane * V + c * VEC;
+            v[c] = *reinterpret_cast<const Vec *>(row + (i >= N ? i - N : i));
+        }
+    }
 #pragma unroll
     for (int c = 0; c < M / VEC; ++c) {
-        const int i = first + c * VEC;
-        const V v = *reinterpret_cast<const V *>(row + (i >= N ? i - N : i));
-        const T *e = reinterpret_cast<const T *>(&v);
+        const T *e = reinterpret_cast<const T *>(&v[c]);
 #pragma unroll
         for (int k = 0; k < VEC; ++k) out[c * VEC + k] = e[k];
     }
 }
 
-// One warp per segment of output cells [out0, out0 + stride) of a row, its 32 V cells
-// from out0 - H on; lane l holds V consecutive ones.  In one pass: the states of the
-// donor sub-steps from the step input (state k from state 0 again for each k: one or
-// two sub-steps in earnest), the sub-steps' transpose in reverse with dL/d dv, and
-// the shift's transpose, g_in[m - K] = sum_u beta_u g'[m + 1 - u].  The shift by K
-// leaves g_in unaligned, so it passes through shared memory to be stored a lane a
-// word.
-//
-// Bound by latency and the launch at 512 x 2048 cells, where a step's 24 bytes a cell
-// stay in L2; the tile passes of k_adj_uniform, with the parameter kernel before
-// them, took 30.6 us there, this 7.3 (FP32, PPM, one or two sub-steps).  A segment a
-// warp, so that few rows still fill the SMs.
+// One segment of k_adj_seg: output cells [out0, out0 + stride) of a row.
 template <typename T, int ORDER>
-__global__ void __launch_bounds__(kSegWarps * 32)
-    k_adj_seg(StepArgs a, const int32_t *row_ids, const RowParams<T> *pars, const T *g_out,
-              T *g_in, T *g_dv)
+__device__ __forceinline__ void adj_segment(const StepArgs &a, const RowInfo &row,
+                                            const RowParams<T> &P, const T (&beta)[6], T *st,
+                                            int out0, int stride, int H, int lane, const T *g_out,
+                                            T *g_in, T *g_dv)
 {
     constexpr int V = kSegV<T>, VEC = 16 / sizeof(T);
     using Vec = typename Vec16<T>::V;
-    __shared__ __align__(16) T stage[kSegWarps][32 * V];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int seg = blockIdx.y * kSegWarps + warp;
-    const int r = row_ids[blockIdx.x];
-    const RowInfo row = a.rows[r];
-    pdl_wait();
-    pdl_trigger();
-    RowParams<T> P;
-    if constexpr (sizeof(T) == 4)
-        shift_params_two_float(a, row, r, seg == 0 && lane == 0, P);
-    else
-        P = pars[r];
     const int N = row.n, nsub = P.nsub;
-    const int H = seg_halo<T>(nsub);
-    const int stride = 32 * V - 2 * H;
-    const int out0 = seg * stride;
-    if (out0 >= N) return;
     const unsigned full = 0xffffffffu;
     const int m0 = out0 - H + lane * V;  // the lane's first cell (may wrap)
-    const int mc = wrap_twice(m0, N);
+    const int mw = wrap_twice(out0 - H, N);  // the warp's first
 
     T g[V];
-    load_cells<T, V>(g_out + row.cell_off, mc, N, g);
-    T beta[6];
-    beta_coeffs<T, ORDER>(P, beta);
+    load_cells<T, V, V>(g_out + row.cell_off, mw, lane, N, g);
     if (nsub > 0) {
         T cp[V + 1], cm[V];  // upwind parts of the faces' Courant numbers (face i: left node)
         {
             T c[V];
-            load_cells<T, V>(static_cast<const T *>(a.dv) + row.cell_off, mc, N, c);
+            load_cells<T, V, V>(static_cast<const T *>(a.dv) + row.cell_off, mw, lane, N, c);
 #pragma unroll
             for (int i = 0; i < V; ++i) {
                 c[i] *= P.cf;
@@ -179,8 +162,8 @@ __global__ void __launch_bounds__(kSegWarps * 32)
             // vector boundary
             const int off = ((-P.K - 1) % VEC + VEC) % VEC;
             T w[V + 3 * VEC];
-            load_cells<T, V + 3 * VEC>(static_cast<const T *>(a.q_in) + row.cell_off,
-                                       wrap_twice(wrap_twice(m0, N) - P.K - 1 - off - VEC, N), N, w);
+            load_cells<T, V + 3 * VEC, V>(static_cast<const T *>(a.q_in) + row.cell_off,
+                                          wrap_twice(mw - P.K - 1 - off - VEC, N), lane, N, w);
 #pragma unroll
             for (int o = 0; o < VEC; ++o)
                 if (o == off) {
@@ -249,7 +232,6 @@ __global__ void __launch_bounds__(kSegWarps * 32)
     for (int i = 0; i < V; ++i) e[i + 2] = g[i];
 #pragma unroll
     for (int i = 0; i < 3; ++i) e[V + 2 + i] = __shfl_down_sync(full, g[i], 1);
-    T *st = stage[warp];
 #pragma unroll
     for (int i = 0; i < V; ++i) {
         T v = T(0);
@@ -264,6 +246,49 @@ __global__ void __launch_bounds__(kSegWarps * 32)
         const int j = out0 + k - P.K;
         gi[j < 0 ? j + N : j] = st[H + k];
     }
+    __syncwarp();  // the stage is free again
+}
+
+// One warp per segment of output cells [out0, out0 + stride) of a row, its 32 V cells
+// from out0 - H on; lane l holds V consecutive ones.  In one pass: the states of the
+// donor sub-steps from the step input (state k from state 0 again for each k: one or
+// two sub-steps in earnest), the sub-steps' transpose in reverse with dL/d dv, and
+// the shift's transpose, g_in[m - K] = sum_u beta_u g'[m + 1 - u].  The shift by K
+// leaves g_in unaligned, so it passes through shared memory to be stored a lane a
+// word.
+//
+// Bound by latency at 512 x 2048 cells, where a step's 24 bytes a cell stay in L2:
+// steps back to back, one or two sub-steps, PPM, 28.6 us with the tile passes of
+// k_adj_uniform and the parameter kernel before them, 8.7 so (FP32; FP64 103 and 63).
+// A segment a warp, so that few rows still fill the SMs; registers capped for six
+// CTAs an SM in FP32 (9.25 us uncapped).
+template <typename T, int ORDER>
+__global__ void __launch_bounds__(kSegWarps * 32, sizeof(T) == 4 ? 6 : 4)
+    k_adj_seg(StepArgs a, const int32_t *row_ids, const RowParams<T> *pars, const T *g_out,
+              T *g_in, T *g_dv)
+{
+    constexpr int V = kSegV<T>;
+    __shared__ __align__(16) T stage[kSegWarps][32 * V];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int seg0 = blockIdx.y * kSegWarps + warp;
+    const int r = row_ids[blockIdx.x];
+    const RowInfo row = a.rows[r];
+    pdl_wait();
+    pdl_trigger();
+    RowParams<T> P;
+    if constexpr (sizeof(T) == 4)
+        shift_params_two_float(a, row, r, seg0 == 0 && lane == 0, P);
+    else
+        P = pars[r];
+    const int N = row.n, nsub = P.nsub;
+    const int H = seg_halo<T>(nsub);
+    const int stride = 32 * V - 2 * H;
+    T beta[6];
+    beta_coeffs<T, ORDER>(P, beta);
+    // one segment a warp, unless the row has more than a grid can
+    for (int64_t seg = seg0; seg * stride < N; seg += (int64_t)gridDim.y * kSegWarps)
+        adj_segment<T, ORDER>(a, row, P, beta, stage[warp], (int)(seg * stride), stride, H, lane,
+                              g_out, g_in, g_dv);
 }
 
 template <typename T, int ORDER>
@@ -463,11 +488,10 @@ cudaError_t launch_adj_t(const Plan &p, const StepArgs &a, const void *g_out, vo
                                           g_out, g_in, g_dv, s);
     const std::vector<int32_t> &rows = p.rows_seg_h[d][ORDER];
     if (!rows.empty()) {
-        int n = 0;
-        for (int32_t r : rows) n = n > p.rows_h[r].n ? n : p.rows_h[r].n;
         // segments of the longest row at the widest halo; the warps past a row's end leave
         const int stride = 32 * kSegV<T> - 2 * seg_halo<T>(a.dv ? RAM_MAX_NSUB : 0);
-        const int y = ((n + stride - 1) / stride + kSegWarps - 1) / kSegWarps;
+        const int segs = (p.seg_nmax[d][ORDER] + stride - 1) / stride;
+        const int y = std::min((segs + kSegWarps - 1) / kSegWarps, 65535);
         cudaError_t e = launch_pdl(k_adj_seg<T, ORDER>, dim3((unsigned)rows.size(), y),
                                    dim3(kSegWarps * 32), 0, s, a,
                                    static_cast<const int32_t *>(p.rows_seg[d][ORDER]),
