@@ -275,8 +275,8 @@ typedef struct {
                                            issue their copies, its shift parameters
                                            formed in the kernel (no parameter kernel
                                            when every row takes it; the default) */
-    int32_t seg_warps;                  /* warp-segment kernel: warps per row CTA, 3..8
-                                           (default 3) */
+    int32_t seg_warps;                  /* warp-segment kernel, FP32: warps per row CTA,
+                                           3..8 (a new plan: 3, more for few long rows) */
     int32_t nonuniform_kernel_f32;      /* FP32 rows with their own mesh: 0 = the
                                            per-order kernels (shared-memory-free without
                                            a residual, tiled with one), 1 = the

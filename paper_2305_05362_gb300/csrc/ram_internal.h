@@ -182,6 +182,7 @@ struct Plan {
     int32_t ncap_fit[2][5] = {{0}};
     // uniform rows taken by the warp-segment kernel, and the tiles of the others
     std::vector<int32_t> rows_seg_h[2][5];
+    int32_t seg_nmax[2][5] = {{0}};  // cells of the longest of them
     std::vector<Tile> tiles_rest_seg_h[2][5];
     // longest and shortest FP32 warp-segment row, by order (the streaming kernel
     // takes the same rows)
@@ -264,7 +265,7 @@ cudaError_t launch_adjoint_nu(const Plan &p, ram_dtype dt, const StepArgs &a, co
 cudaError_t launch_rows(const Plan &p, ram_dtype dt, const StepArgs &a, cudaStream_t s,
                         int order, const RowPos *rows, int n_rows, int ncap);
 cudaError_t launch_useg(const Plan &p, ram_dtype dt, const StepArgs &a, cudaStream_t s,
-                        int order, const int32_t *row_ids, int n_rows);
+                        int order, const int32_t *row_ids, int n_rows, int longest);
 
 // streaming kernel for the FP32 warp-segment rows of one order (ram_stream.cu)
 cudaError_t launch_stream(const Plan &p, const StepArgs &a, cudaStream_t s, int order);

@@ -142,6 +142,6 @@ extern "C" ram_status ram_step_uniform_noalloc(ram_dtype dtype, int32_t n_rows,
     a.limiter = (flags & RAM_LIMITER_OFF) ? 0 : 1;
     a.err = device_errors ? reinterpret_cast<int *>(device_errors) : err;
     cudaError_t e = launch_params(p, dtype, a, s);
-    if (e == cudaSuccess) e = launch_useg(p, dtype, a, s, order, ids, n_rows);
+    if (e == cudaSuccess) e = launch_useg(p, dtype, a, s, order, ids, n_rows, n);
     return e == cudaSuccess ? RAM_OK : RAM_ERR_CUDA;
 }

@@ -224,6 +224,29 @@ void general_caps(const Plan &p, std::vector<Tile> &tl, int32_t &whole, int32_t 
     }
 }
 
+// Warps per row CTA of the FP32 ring kernel (24 resident warps an SM).  Three fill
+// the SMs best when the rows do (1024 rows of 4096 cells: 14.6 us, 16.4 with four,
+// 17.5 with eight: the rows' last segments are dealt out more evenly over smaller
+// CTAs).  Fewer rows leave SMs idle: then the fewest warps, within what is resident
+// together, that take a row in the fewest rounds of segments (us per step with three
+// and with the choice: 32 x 16384 cells 21.2, 13.0; 150 x 8192 12.1, 8.1; 300 x 8192
+// 13.3, 10.1; 512 x 4096 10.1, 9.5; 512 x 2048 6.3, 6.4; 128 x 1024 3.7, 3.1).
+int default_seg_warps(const Plan &p)
+{
+    int rows = 0, longest = 0;
+    for (int o = 2; o <= 4; ++o) {
+        rows += (int)p.rows_seg_h[0][o].size();
+        longest = std::max(longest, p.seg_nmax[0][o]);
+    }
+    if (rows == 0) return 3;
+    const int most = std::min(std::max(p.sm_count * 24 / rows, 3), 8);
+    const int segments = (longest + 247) / 248;
+    int best = 3;
+    for (int w = 4; w <= most; ++w)
+        if ((segments + w - 1) / w < (segments + best - 1) / best) best = w;
+    return best;
+}
+
 }  // namespace
 
 // Split every row into near-equal tiles of at most tile_cells output cells and
@@ -246,6 +269,7 @@ ram_status build_tiles(Plan &p)
             p.tiles_rest_h[d][o].clear();
             p.ncap_fit[d][o] = 0;
             p.rows_seg_h[d][o].clear();
+            p.seg_nmax[d][o] = 0;
             p.tiles_rest_seg_h[d][o].clear();
             if (d == 0) {
                 p.stream_nmax[o] = 0;
@@ -291,6 +315,7 @@ ram_status build_tiles(Plan &p)
                     if (seg) {
                         if (t == 0) {
                             p.rows_seg_h[d][ri.order].push_back(r);
+                            p.seg_nmax[d][ri.order] = std::max(p.seg_nmax[d][ri.order], n);
                             if (d == 0) {
                                 p.stream_nmax[ri.order] = std::max(p.stream_nmax[ri.order], n);
                                 p.stream_nmin[ri.order] = p.stream_nmin[ri.order] == 0
@@ -463,10 +488,9 @@ extern "C" ram_status ram_plan_mesh(const ram_mesh_desc *desc, int device, ram_p
     p->n_cells = ro[nr];
     p->flags = desc->flags;
     p->limiter = (desc->flags & RAM_LIMITER_OFF) ? 0 : 1;
-    // FP32 warp-segment rows default to the shared-memory ring form, 3 warps per
-    // row CTA (the fastest measured on the disks; the autotuner may change it)
+    // FP32 warp-segment rows default to the shared-memory ring form (the fastest
+    // measured on the disks; the autotuner may change it)
     p->seg_variant = 2;
-    p->seg_warps = 3;
     p->row_offset.assign(ro, ro + nr + 1);
     p->adj_all = ((desc->flags & RAM_ADJOINT) && p->limiter) ? 1 : 0;
     const size_t n_nodes = shared ? (size_t)(ro[1] + 1) : (size_t)(ro[nr] + nr);
@@ -583,6 +607,7 @@ extern "C" ram_status ram_plan_mesh(const ram_mesh_desc *desc, int device, ram_p
             st = RAM_ERR_NOMEM;
     }
     if (st == RAM_OK) st = build_tiles(*p);
+    if (st == RAM_OK) p->seg_warps = default_seg_warps(*p);
     if (st == RAM_OK && cudaDeviceSynchronize() != cudaSuccess) st = RAM_ERR_CUDA;
     if (st != RAM_OK) {
         free_device(*p);

@@ -200,7 +200,7 @@ cudaError_t launch_order(const Plan &p, const StepArgs &a, cudaStream_t s)
     }
     if (p.uniform_kernel[d] == 1 && !p.rows_seg_h[d][ORDER].empty()) {
         cudaError_t e = launch_useg(p, dt, a, s, ORDER, p.rows_seg[d][ORDER],
-                                    (int)p.rows_seg_h[d][ORDER].size());
+                                    (int)p.rows_seg_h[d][ORDER].size(), p.seg_nmax[d][ORDER]);
         if (e != cudaSuccess) return e;
         return launch_tiles<T, ORDER>(p, a, s, p.tiles_rest_seg[d][ORDER],
                                       p.tiles_rest_seg_h[d][ORDER]);

@@ -14,6 +14,7 @@
 // overlap by 2*H4 cells and each stores only its interior.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -63,10 +64,10 @@ __device__ __forceinline__ void seg_row(const StepArgs &a, const RowParams<T> &P
     S.off = ((-P.K - 1) % VEC + VEC) % VEC;
 }
 
-// Segment seg of a row: this lane's V cells.
+// Output cells [out0, out0 + S.stride) of a row, those below `end`: this lane's V cells.
 template <typename T, int ORDER, int V, bool LIM, bool VL>
-__device__ __forceinline__ void seg_step(const RowParams<T> &P, const SegRow<T> &S, int seg,
-                                         int lane, T &cmax)
+__device__ __forceinline__ void seg_step(const RowParams<T> &P, const SegRow<T> &S, int out0,
+                                         int end, int lane, T &cmax)
 {
     static_assert(V % (16 / sizeof(T)) == 0, "V must be a whole number of 16-byte vectors");
     constexpr int VEC = 16 / sizeof(T);
@@ -77,7 +78,6 @@ __device__ __forceinline__ void seg_step(const RowParams<T> &P, const SegRow<T> 
     T *qout = S.qout;
     constexpr bool lim = LIM;
     constexpr bool vl = VL;
-    const int out0 = seg * stride;               // first output cell of the segment
     const int m0 = out0 - H4 + lane * V;         // this lane's first cell (may wrap)
     // ---- source window: cells p0-2 .. p0+V+2, p0 = m0 - K - 1 ----
     const int p0 = m0 - P.K - 1;
@@ -210,14 +210,14 @@ __device__ __forceinline__ void seg_step(const RowParams<T> &P, const SegRow<T> 
         }
     }
 
-    // ---- store the interior [H4, H4 + stride) of the segment, cells < N ----
-    // H4, stride, out0 and N are whole vectors, so every vector of the lane is
+    // ---- store the interior [H4, H4 + stride) of the segment, cells < end ----
+    // H4, stride, out0 and end are whole vectors, so every vector of the lane is
     // either wholly stored or wholly halo: no scalar tail
     const int li0 = lane * V;                    // local index of cur[0]
 #pragma unroll
     for (int c = 0; c < V / VEC; ++c) {
         const int li = li0 + c * VEC;
-        if (li >= H4 && li < H4 + stride && m0 + c * VEC < N) {
+        if (li >= H4 && li < H4 + stride && m0 + c * VEC < end) {
             Vec vv;
             if (sizeof(T) == 4) {
                 float4 f4 = make_float4((float)cur[c * VEC], (float)cur[c * VEC + 1],
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(256, V * sizeof(T) <= 32 ? 3 : 2)
     seg_row<T, V, VL>(a, P, S);
     T cmax = T(0);
     for (int seg = warp; seg < S.nseg; seg += nwarps)
-        seg_step<T, ORDER, V, LIM, VL>(P, S, seg, lane, cmax);
+        seg_step<T, ORDER, V, LIM, VL>(P, S, seg * S.stride, S.N, lane, cmax);
     if (cmax > T(1)) atomicOr(a.err, ERR_CFL);
 }
 
@@ -563,6 +563,263 @@ __global__ void __launch_bounds__(256, 3)
     if (cmax > 1.0f) atomicOr(a.err, ERR_CFL);
 }
 
+// ---------------------------------------------------------------------------
+// FP64 rows
+// ---------------------------------------------------------------------------
+// The FP64 pipe takes a warp instruction every 16 cycles of an SM (64 of a
+// scheduler), the integer pipe 32 times as many: the form below spends FP64
+// instructions on sums and products only.  Comparisons, signs, minima of magnitudes
+// and scalings by powers of two work on the bits (a magnitude's order is its bits'),
+// quotients are a cubic Newton step from the hardware's reciprocal approximation (3
+// FP64 instructions and the product, against about ten for a range-checked divide;
+// within 1 ulp), and nothing is formed twice (lanes share slopes, partials and
+// fluxes).  About 10 FP64 instructions a cell for the limited PPM remap and 11 a van
+// Leer sub-step; before, 91 in all on the 1024 x 4096 disk.
+// Subnormal differences count as zero here.  A warp whose window or dv holds a value
+// of 2^1000 or more in magnitude, an infinity or a NaN, or whose whole window is below
+// 2^-400, takes the compare-and-select form (seg_step) for its segment: infinities and
+// NaN travel as in IEEE arithmetic, and the products of tiny differences that decide
+// the limiters vanish there, as they do in the other uniform-row kernels.
+
+__device__ __forceinline__ unsigned long long mag(double x)
+{
+    return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+// magnitude times 2^k, k = 1 or 2 (subnormals: 0)
+__device__ __forceinline__ unsigned long long mag_up(unsigned long long m, int k)
+{
+    return (m >> 52) == 0 ? 0ull : m + ((unsigned long long)k << 52);
+}
+__device__ __forceinline__ unsigned long long mag_min(unsigned long long a, unsigned long long b)
+{
+    return a < b ? a : b;
+}
+// the magnitude m with s's sign, zero where s and t differ in sign
+__device__ __forceinline__ double mag_signed(unsigned long long m, double s, double t)
+{
+    const int hs = __double2hiint(s), ht = __double2hiint(t);
+    const unsigned long long v = m | ((unsigned long long)(hs & 0x80000000) << 32);
+    return (hs ^ ht) < 0 ? 0.0 : __longlong_as_double((long long)v);
+}
+__device__ __forceinline__ double half_of(double x)
+{
+    const long long b = __double_as_longlong(x);
+    return ((b >> 52) & 0x7ff) < 2 ? 0.0 : __longlong_as_double(b - (1ll << 52));
+}
+// half the van Leer slope, dl dr / (dl + dr) where dl and dr have one sign, else 0
+__device__ __forceinline__ double half_vl_bits(double dl, double dr)
+{
+    const double p = dl * dr, s = dl + dr;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(s));
+    const double e = fma(-s, r, 1.0);
+    const double u = p * r;
+    const double h = fma(u, fma(e, e, e), u);
+    const bool one_sign = (__double2hiint(dl) ^ __double2hiint(dr)) >= 0;
+    // s normal: both zero, or sums too small for the reciprocal, have no slope
+    return one_sign && (mag(s) >> 52) > 1 ? h : 0.0;
+}
+// the high word of a magnitude (ordered as the magnitudes are), and its bounds above
+__device__ __forceinline__ unsigned mag_hi(double x)
+{
+    return (unsigned)__double2hiint(x) & 0x7fffffffu;
+}
+constexpr unsigned kMagBig = 0x7e700000u;    // 2^1000; infinity and NaN above
+constexpr unsigned kMagSmall = 0x26f00000u;  // 2^-400
+
+// The segment's cells in the compare-and-select form, 4 a lane.
+template <int ORDER, bool LIM, bool VL>
+__device__ __noinline__ void seg_step_f64_any(const StepArgs &a, const RowParams<double> &P, int out0,
+                                              int end, int lane, double *cmax)
+{
+    SegRow<double> S;
+    seg_row<double, 4, VL>(a, P, S);
+    for (int o = out0; o < end; o += S.stride)
+        seg_step<double, ORDER, 4, LIM, VL>(P, S, o, end, lane, *cmax);
+}
+
+// One segment of k_useg_f64: output cells [out0, out0 + stride) of a row, 8 a lane.
+template <int ORDER, bool LIM, bool VL>
+__device__ __forceinline__ void seg_f64(const StepArgs &a, const RowParams<double> &P, bool has_dv,
+                                        int out0, int stride, int HL, int lane)
+{
+    constexpr int V = 8, VEC = 2, NW = V + 3 * VEC;
+    const int N = P.n, nsub = P.nsub;
+    const int end = min(out0 + stride, N);
+    const unsigned full = 0xffffffffu;
+    const int m0 = out0 - HL + lane * V;
+    const double *qin = static_cast<const double *>(a.q_in) + P.cell_off;
+    const int off = ((-P.K - 1) % VEC + VEC) % VEC;
+    double w[NW], c[V];
+    bool other = false;
+    unsigned top = 0;
+    {
+        const int b0 = wrap2(wrap2(m0, N) - P.K - 1 - off - VEC, N);
+#pragma unroll
+        for (int k = 0; k < NW / VEC; ++k) {
+            const double2 v = *reinterpret_cast<const double2 *>(qin + wrap1(b0 + k * VEC, N));
+            w[2 * k] = v.x;
+            w[2 * k + 1] = v.y;
+        }
+    }
+    if (has_dv) {
+        const double *dvp = static_cast<const double *>(a.dv) + P.cell_off;
+        const int b0 = wrap2(m0, N);
+#pragma unroll
+        for (int k = 0; k < V / VEC; ++k) {
+            const double2 v = *reinterpret_cast<const double2 *>(dvp + wrap1(b0 + k * VEC, N));
+            c[2 * k] = v.x;
+            c[2 * k + 1] = v.y;
+        }
+#pragma unroll
+        for (int i = 0; i < V; ++i) other |= mag_hi(c[i]) >= kMagBig;
+    }
+#pragma unroll
+    for (int k = 0; k < NW; ++k) top = max(top, mag_hi(w[k]));
+    top = __reduce_max_sync(full, top);
+    if (__any_sync(full, other) || top >= kMagBig || (top < kMagSmall && top > 0)) {
+        double cm = 0.0;
+        seg_step_f64_any<ORDER, LIM, VL>(a, P, out0, end, lane, &cm);
+        if (cm > 1.0) atomicOr(a.err, ERR_CFL);
+        return;
+    }
+    // ---- the remap: q[j] is source cell p - 2 + j, p = m0 - K - 1 ----
+    double q[V + 4];
+#pragma unroll
+    for (int j = 0; j < V + 4; ++j) q[j] = off ? w[j + 1] : w[j];
+    double cur[V];
+    if (P.whole) {
+#pragma unroll
+        for (int k = 0; k < V; ++k) cur[k] = q[k + 3];
+    } else {
+        double A[V + 1];  // left partials of the lane's own source cells p .. p + V - 1
+        if (ORDER == 3) {
+            // remap_warp3's form of App. A
+            double dif[V + 1], Dq[V + 2];
+#pragma unroll
+            for (int i = 0; i <= V; ++i) dif[i] = q[i + 2] - q[i + 1];
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                const double D = dif[j] + dif[j + 1];
+                Dq[j + 1] = LIM ? mag_signed(mag_min(mag(D), mag_up(mag_min(mag(dif[j]), mag(dif[j + 1])), 2)),
+                                             dif[j], dif[j + 1])
+                                : D;
+            }
+            Dq[0] = __shfl_up_sync(full, Dq[V], 1);
+            Dq[V + 1] = __shfl_down_sync(full, Dq[1], 1);
+            const double xi = P.c[3], cR = P.c[1], cL = P.c[0];
+            double El = Dq[1] - Dq[0];
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                const double Er = Dq[j + 2] - Dq[j + 1];
+                double fa = fma(Er, -1.0 / 12.0, half_of(dif[j + 1]));
+                double fb = fma(El, 1.0 / 12.0, half_of(dif[j]));
+                if (LIM) {
+                    const unsigned long long ma = mag(fa), mb = mag(fb);
+                    const double a1 = mag_signed(mag_min(ma, mag_up(mb, 1)), fa, fb);
+                    fb = mag_signed(mag_min(mb, mag_up(ma, 1)), fb, fa);
+                    fa = a1;
+                }
+                A[j] = fma(xi, q[j + 2], fma(cR, fa, -cL * fb));
+                El = Er;
+            }
+        } else if (ORDER == 2) {
+            double dn = q[2] - q[1];
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                const double up = q[j + 3] - q[j + 2];
+                // the slope: twice half_vl, or the centred one
+                const double h = LIM ? half_vl_bits(dn, up) : dn + up;
+                A[j] = fma(q[j + 2], P.c[0], h * (LIM ? 2.0 * P.c[1] : 0.5 * P.c[1]));
+                dn = up;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < V; ++j)
+                A[j] = fma(P.c[0], q[j],
+                           fma(P.c[1], q[j + 1],
+                               fma(P.c[2], q[j + 2], fma(P.c[3], q[j + 3], P.c[4] * q[j + 4]))));
+        }
+        A[V] = __shfl_down_sync(full, A[0], 1);
+#pragma unroll
+        for (int k = 0; k < V; ++k) cur[k] = (q[k + 2] - A[k]) + A[k + 1];
+    }
+    // ---- residual sub-steps (residual_group_cs's flux, each formed once) ----
+    if (has_dv) {
+        double wc[V];  // the swept part's midpoint: +-1 - c
+        bool bad = false;
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            c[i] *= P.cf;
+            bad |= mag(c[i]) > 0x3ff0000000000000ull;  // |c| > 1
+            if (VL) wc[i] = (__double_as_longlong(c[i]) > 0 ? 1.0 : -1.0) - c[i];
+        }
+        if (bad) atomicOr(a.err, ERR_CFL);
+        for (int sub = 0; sub < nsub; ++sub) {
+            const double zl = __shfl_up_sync(full, cur[V - 1], 1);
+            double F[V + 1];
+            if (VL) {
+                const double zr = __shfl_down_sync(full, cur[0], 1);
+                double h[V], dl = cur[0] - zl;
+#pragma unroll
+                for (int i = 0; i < V; ++i) {
+                    const double dr = (i < V - 1 ? cur[i + 1] : zr) - cur[i];
+                    h[i] = half_vl_bits(dl, dr);
+                    dl = dr;
+                }
+                const double hl = __shfl_up_sync(full, h[V - 1], 1);
+#pragma unroll
+                for (int i = 0; i < V; ++i) {
+                    const bool pos = __double_as_longlong(c[i]) > 0;
+                    const double zu = pos ? (i ? cur[i - 1] : zl) : cur[i];
+                    const double hu = pos ? (i ? h[i - 1] : hl) : h[i];
+                    F[i] = c[i] * fma(hu, wc[i], zu);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < V; ++i)
+                    F[i] = c[i] * (__double_as_longlong(c[i]) > 0 ? (i ? cur[i - 1] : zl) : cur[i]);
+            }
+            F[V] = __shfl_down_sync(full, F[0], 1);
+#pragma unroll
+            for (int i = 0; i < V; ++i) cur[i] -= F[i + 1] - F[i];
+        }
+    }
+    double *qout = static_cast<double *>(a.q_out) + P.cell_off;
+#pragma unroll
+    for (int k = 0; k < V / VEC; ++k) {
+        const int li = lane * V + k * VEC, m = m0 + k * VEC;
+        if (li >= HL && m < end)
+            *reinterpret_cast<double2 *>(qout + m) = make_double2(cur[2 * k], cur[2 * k + 1]);
+    }
+}
+
+// One warp per segment, 8 cells a lane; the row's parameters come from the parameter
+// kernel.  Few warps keep the FP64 pipe busy, so registers are plentiful; a segment a
+// warp (not a row a CTA) spreads rows of unequal sub-step counts over the SMs.
+// Bound by the FP64 pipe.
+template <int ORDER, bool LIM, bool VL>
+__global__ void __launch_bounds__(128, 3)
+    k_useg_f64(StepArgs a, const int32_t *row_ids, const RowParams<double> *pars)
+{
+    constexpr int V = 8;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int r = row_ids[blockIdx.x];
+    pdl_wait();
+    const RowParams<double> P = pars[r];
+    const int N = P.n, nsub = P.nsub;
+    const bool has_dv = (a.mode != MODE_SHIFT) && (a.dv != nullptr) && nsub > 0;
+    // halo, whole vectors: the sub-steps spoil nsub (donor) or 2 nsub cells at each end,
+    // the remap with shared neighbours one on the right, the PPM one one more on each side
+    const int spoil = nsub * (VL ? 2 : 1);
+    const int HL = (spoil + (ORDER == 3 ? 1 : 0) + 1) / 2 * 2;
+    const int HR = (spoil + (ORDER == 3 ? 2 : 1) + 1) / 2 * 2;
+    const int stride = 32 * V - HL - HR;
+    // one segment a warp, unless the row has more than a grid can
+    for (int64_t seg = blockIdx.y * 4 + warp; seg * stride < N; seg += (int64_t)gridDim.y * 4)
+        seg_f64<ORDER, LIM, VL>(a, P, has_dv, (int)(seg * stride), stride, HL, lane);
+}
+
 template <typename T, int ORDER, int V>
 cudaError_t launch_useg_v(const StepArgs &a, cudaStream_t s, int threads, const int32_t *row_ids,
                           int n_rows,
@@ -622,6 +879,22 @@ cudaError_t launch_useg_ring(const Plan &p, const StepArgs &a, cudaStream_t s, i
     return launch_ring_k<ORDER, V, false, false>(p, a, s, threads, row_ids, n_rows);
 }
 
+// `longest`: cells of the longest row.
+template <int ORDER>
+cudaError_t launch_useg_f64(const StepArgs &a, cudaStream_t s, const int32_t *row_ids, int n_rows,
+                            int longest, const RowParams<double> *par)
+{
+    const bool lim = a.limiter != 0, vl = a.scheme == RAM_VANLEER;
+    // segments at the widest halo; the warps past a row's end leave
+    const int most = a.mode != MODE_SHIFT && a.dv != nullptr ? RAM_MAX_NSUB * (vl ? 2 : 1) : 0;
+    const int stride = 256 - (most + 2) / 2 * 2 - (most + 3) / 2 * 2;
+    const dim3 grid(n_rows, std::min(((longest + stride - 1) / stride + 3) / 4, 65535));
+    void (*kern)(StepArgs, const int32_t *, const RowParams<double> *) =
+        lim ? (vl ? k_useg_f64<ORDER, true, true> : k_useg_f64<ORDER, true, false>)
+            : (vl ? k_useg_f64<ORDER, false, true> : k_useg_f64<ORDER, false, false>);
+    return launch_pdl(kern, grid, dim3(128), 0, s, a, row_ids, par);
+}
+
 template <int ORDER>
 cudaError_t launch_useg_f32(const Plan &p, const StepArgs &a, cudaStream_t s, int threads,
                             const int32_t *row_ids, int n_rows, const RowParams<float> *par)
@@ -641,7 +914,7 @@ cudaError_t launch_useg_f32(const Plan &p, const StepArgs &a, cudaStream_t s, in
 // flight per warp, 1 the next segment's loads in flight in registers, 2 a ring of
 // shared-memory stages per warp (with the shift parameters formed in the kernel).
 cudaError_t launch_useg(const Plan &p, ram_dtype dt, const StepArgs &a, cudaStream_t s,
-                        int order, const int32_t *row_ids, int n_rows)
+                        int order, const int32_t *row_ids, int n_rows, int longest)
 {
     if (n_rows == 0) return cudaSuccess;
     // warps per row CTA: a row's segments take ceil(segments / warps) rounds and the
@@ -654,9 +927,9 @@ cudaError_t launch_useg(const Plan &p, ram_dtype dt, const StepArgs &a, cudaStre
         if (order == 3) return launch_useg_f32<3>(p, a, s, threads, row_ids, n_rows, pf);
         return launch_useg_f32<4>(p, a, s, threads, row_ids, n_rows, pf);
     }
-    if (order == 2) return launch_useg_v<double, 2, 4>(a, s, threads, row_ids, n_rows, pd);
-    if (order == 3) return launch_useg_v<double, 3, 4>(a, s, threads, row_ids, n_rows, pd);
-    return launch_useg_v<double, 4, 4>(a, s, threads, row_ids, n_rows, pd);
+    if (order == 2) return launch_useg_f64<2>(a, s, row_ids, n_rows, longest, pd);
+    if (order == 3) return launch_useg_f64<3>(a, s, row_ids, n_rows, longest, pd);
+    return launch_useg_f64<4>(a, s, row_ids, n_rows, longest, pd);
 }
 
 }  // namespace ram
