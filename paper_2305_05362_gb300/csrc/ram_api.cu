@@ -67,13 +67,13 @@ StepArgs base_args(const Plan *p, const void *q_in, void *q_out)
     return a;
 }
 
-// Every row of this FP32 launch forms its own shift parameters, so no parameter
-// kernel is needed: uniform rows on the shared-memory ring form of the
-// warp-segment kernel (which needs 16-byte aligned arrays), rows with their own
-// mesh on the non-uniform warp-segment kernel.
+// Every row of this launch forms its own shift parameters, so no parameter kernel is
+// needed: FP32 uniform rows on the shared-memory ring form of the warp-segment kernel
+// (which needs 16-byte aligned arrays), rows with their own mesh on the non-uniform
+// warp-segment kernels.
 bool rows_form_params(const Plan &p, ram_dtype dt, const StepArgs &a)
 {
-    if (dt != RAM_F32) return false;
+    if (dt != RAM_F32) return p.nseg_rows == p.n_rows;
     size_t seg = 0;
     if (p.n_uniform_rows > 0) {
         if (p.uniform_kernel[0] != 1 || p.seg_variant != 2) return false;

@@ -627,8 +627,9 @@ __global__ void __launch_bounds__(512)
     }
 }
 
-// A list of non-uniform tiles of one order for the general kernels: every row's
-// (FP64) or the rows the FP32 warp-segment kernel does not take.
+// A list of non-uniform tiles of one order for the general kernels: the rows that the
+// warp-segment kernels do not take, or (FP32 with the tuning's per-order kernels)
+// every row's.
 struct GenList {
     const Tile *tiles;
     int n, whole;
@@ -637,7 +638,7 @@ struct GenList {
 
 GenList gen_list(const Plan &p, int order, bool f32)
 {
-    if (f32 && p.nu_kernel == 1)
+    if (!f32 || p.nu_kernel == 1)
         return {p.tiles_general32[order], (int)p.tiles_general32_h[order].size(),
                 p.gen32_whole[order], p.gen32_wcap[order], p.gen32_qcap[order]};
     return {p.tiles_general[order], (int)p.tiles_general_h[order].size(), p.gen_whole[order],
@@ -747,6 +748,7 @@ cudaError_t launch_general(const Plan &p, ram_dtype dt, const StepArgs &a, cudaS
         if ((e = launch_general_t<float, 3>(p, a, s, launched)) != cudaSuccess) return e;
         return launch_general_t<float, 4>(p, a, s, launched);
     }
+    if ((e = launch_nseg_f64(p, a, s)) != cudaSuccess) return e;
     if ((e = launch_general_t<double, 2>(p, a, s, launched)) != cudaSuccess) return e;
     if ((e = launch_general_t<double, 3>(p, a, s, launched)) != cudaSuccess) return e;
     return launch_general_t<double, 4>(p, a, s, launched);

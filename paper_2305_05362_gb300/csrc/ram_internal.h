@@ -148,9 +148,8 @@ struct Plan {
     int32_t gen_whole[5] = {0};
     int32_t gen_wcap[5][2] = {{0}};  // [order][class]
     int32_t gen_qcap[5][2] = {{0}};
-    // FP32: the tiles of the rows the warp-segment kernel does not take (the same
-    // layout as above), and the warp-segment kernel's tiles (window = cells per
-    // segment of the row) with the largest source window of any of its segments
+    // the tiles of the rows the warp-segment kernels do not take (the same layout as
+    // above)
     std::vector<Tile> tiles_general32_h[5];
     int32_t gen32_whole[5] = {0};
     int32_t gen32_wcap[5][2] = {{0}};
@@ -246,6 +245,8 @@ cudaError_t launch_uniform(const Plan &p, ram_dtype dt, const StepArgs &a, cudaS
 cudaError_t launch_general(const Plan &p, ram_dtype dt, const StepArgs &a, cudaStream_t s);
 // FP32 rows with their own mesh, warp-segment kernel (ram_nseg.cu)
 cudaError_t launch_nseg(const Plan &p, const StepArgs &a, cudaStream_t s);
+// the same rows in FP64 (ram_nseg_f64.cu)
+cudaError_t launch_nseg_f64(const Plan &p, const StepArgs &a, cudaStream_t s);
 cudaError_t launch_row_mass(const Plan &p, ram_dtype dt, const void *q, double *out,
                             cudaStream_t s);
 cudaError_t launch_adjoint(const Plan &p, ram_dtype dt, const StepArgs &a, const void *g_out,

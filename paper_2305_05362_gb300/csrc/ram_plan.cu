@@ -150,6 +150,7 @@ int nseg_cells(const double *x, const double *w, int n, int &qs)
     if (n < kNsegMinCells) return 0;
     const int room = kNsegWin - 2 * kNsegHR;
     const double L = x[n] - x[0];
+    if (!(L > 1e-250 && L < 1e250)) return 0;  // widths are scaled by their exponents
     double w_min = w[0], w_max = w[0], reach = 2.0 * L;
     for (int i = 1; i < n; ++i) {
         w_min = std::min(w_min, w[i]);

@@ -18,6 +18,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "ram_bits.cuh"
 #include "ram_lane.cuh"
 #include "ram_tma.cuh"
 
@@ -580,52 +581,6 @@ __global__ void __launch_bounds__(256, 3)
 // 2^-400, takes the compare-and-select form (seg_step) for its segment: infinities and
 // NaN travel as in IEEE arithmetic, and the products of tiny differences that decide
 // the limiters vanish there, as they do in the other uniform-row kernels.
-
-__device__ __forceinline__ unsigned long long mag(double x)
-{
-    return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
-}
-// magnitude times 2^k, k = 1 or 2 (subnormals: 0)
-__device__ __forceinline__ unsigned long long mag_up(unsigned long long m, int k)
-{
-    return (m >> 52) == 0 ? 0ull : m + ((unsigned long long)k << 52);
-}
-__device__ __forceinline__ unsigned long long mag_min(unsigned long long a, unsigned long long b)
-{
-    return a < b ? a : b;
-}
-// the magnitude m with s's sign, zero where s and t differ in sign
-__device__ __forceinline__ double mag_signed(unsigned long long m, double s, double t)
-{
-    const int hs = __double2hiint(s), ht = __double2hiint(t);
-    const unsigned long long v = m | ((unsigned long long)(hs & 0x80000000) << 32);
-    return (hs ^ ht) < 0 ? 0.0 : __longlong_as_double((long long)v);
-}
-__device__ __forceinline__ double half_of(double x)
-{
-    const long long b = __double_as_longlong(x);
-    return ((b >> 52) & 0x7ff) < 2 ? 0.0 : __longlong_as_double(b - (1ll << 52));
-}
-// half the van Leer slope, dl dr / (dl + dr) where dl and dr have one sign, else 0
-__device__ __forceinline__ double half_vl_bits(double dl, double dr)
-{
-    const double p = dl * dr, s = dl + dr;
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(s));
-    const double e = fma(-s, r, 1.0);
-    const double u = p * r;
-    const double h = fma(u, fma(e, e, e), u);
-    const bool one_sign = (__double2hiint(dl) ^ __double2hiint(dr)) >= 0;
-    // s normal: both zero, or sums too small for the reciprocal, have no slope
-    return one_sign && (mag(s) >> 52) > 1 ? h : 0.0;
-}
-// the high word of a magnitude (ordered as the magnitudes are), and its bounds above
-__device__ __forceinline__ unsigned mag_hi(double x)
-{
-    return (unsigned)__double2hiint(x) & 0x7fffffffu;
-}
-constexpr unsigned kMagBig = 0x7e700000u;    // 2^1000; infinity and NaN above
-constexpr unsigned kMagSmall = 0x26f00000u;  // 2^-400
 
 // The segment's cells in the compare-and-select form, 4 a lane.
 template <int ORDER, bool LIM, bool VL>
