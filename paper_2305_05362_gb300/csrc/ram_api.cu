@@ -101,12 +101,28 @@ ram_status run(const Plan *p, ram_dtype dt, const StepArgs &a0, void *stream)
     return e == cudaSuccess ? RAM_OK : RAM_ERR_CUDA;
 }
 
-// A step of an A4 plan: corrected averages of the input, the shift of them,
+// A step of an A4 plan whose rows all take a warp-segment kernel is one launch of it,
+// which forms the averages and recovers the point values in registers.
+bool a4_in_kernel(const Plan &p, ram_dtype dt, const StepArgs &a)
+{
+    const int d = dt == RAM_F32 ? 0 : 1;
+    if (p.uniform_kernel[d] != 1 || (d == 0 && p.seg_variant != 2)) return false;
+    for (const void *ptr : {a.q_in, static_cast<const void *>(a.q_out), a.dv})
+        if ((uintptr_t)ptr % 16) return false;
+    return p.rows_seg_h[d][3].size() == (size_t)p.n_rows;
+}
+
+// A step of an A4 plan in general: corrected averages of the input, the shift of them,
 // point values back, then the residual step (if any) on the point values.
 ram_status run_a4(const Plan *p, ram_dtype dt, const StepArgs &a0, void *stream)
 {
     DeviceGuard g(p->device);
     if (!g.ok) return RAM_ERR_CUDA;
+    if (a4_in_kernel(*p, dt, a0)) {
+        StepArgs a = a0;
+        a.a4 = 1;
+        return run(p, dt, a, stream);
+    }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     char *s1 = static_cast<char *>(p->a4_scratch);
     char *s2 = s1 + (size_t)p->n_cells * sizeof(double);

@@ -109,6 +109,7 @@ struct StepArgs {
     const Density *density; // mesh-density functions of rows that have one
     const uint32_t *x32;    // xfix >> qshift, the low 32 bits (warp-segment rows)
     uint32_t wait_limit = kWaitLimit;  // tries of every bounded mbarrier wait
+    int32_t a4 = 0;         // the cells are point values (RAM_A4), corrected in the kernel
     int32_t row_phase = 0;  // no parameter kernel ran: the row kernels advance the phase
 };
 

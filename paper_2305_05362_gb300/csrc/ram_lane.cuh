@@ -162,6 +162,62 @@ __device__ __forceinline__ void remap_warp3(const float (&q)[V + 5], const RowPa
     for (int k = 0; k < V; ++k) out[k] = (q[k + 2] - A[k]) + A[k + 1];
 }
 
+// ---- the fourth-order cell-average correction (Sec. 3.1) in a warp's registers ----
+// r: the root of r^2 + 22 r + 1 = 0 inside the unit circle.  22 Q_i + Q_{i-1} + Q_{i+1} =
+// -(1/r) (1 - r S)(1 - r S^-1) Q with S the shift by one cell, so that the averages'
+// inverse is two first-order recursions, one each way.
+constexpr double kA4Root = -0.04554884989667805;
+// cells of a warp's range that a missing neighbour spoils at each end: r^8 < 2e-11 in
+// FP32, r^14 < 2e-19 in FP64 (of the neighbours' values)
+template <typename T> constexpr int kA4Halo = sizeof(T) == 4 ? 8 : 14;
+
+// q[1 .. M-2] to averages, q_i + (q_{i+1} - 2 q_i + q_{i-1}) / 24
+template <typename T, int M> __device__ __forceinline__ void a4_average(T (&q)[M])
+{
+    T left = q[0];
+#pragma unroll
+    for (int i = 1; i < M - 1; ++i) {
+        const T c = q[i];
+        q[i] = fma(q[i + 1] - T(2) * c + left, T(1) / T(24), c);
+        left = c;
+    }
+}
+
+// Averages of the lane's V consecutive cells to point values: Q = <Q> - M^-1 (D <Q>) / 24
+// with D the second difference and M = 1 + D / 24, so that the recursions run on the
+// small D <Q> and their rounding with it; M^-1 / 24 = -r times the two recursions.  A
+// lane's starts with what its neighbours' bring: the next lane's alone (r^V of the one
+// beyond: below FP32 rounding for V = 8), in FP64 the next two.
+template <typename T, int V> __device__ __forceinline__ void a4_points(T (&x)[V])
+{
+    const unsigned full = 0xffffffffu;
+    const T r = (T)kA4Root;
+    T rp[V];
+    rp[0] = r;
+#pragma unroll
+    for (int i = 1; i < V; ++i) rp[i] = rp[i - 1] * r;
+    T t[V], d = x[0] - __shfl_up_sync(full, x[V - 1], 1);
+    const T xr = __shfl_down_sync(full, x[0], 1);
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+        const T e = (i < V - 1 ? x[i + 1] : xr) - x[i];
+        t[i] = e - d;
+        d = e;
+    }
+#pragma unroll
+    for (int i = 1; i < V; ++i) t[i] = fma(r, t[i - 1], t[i]);
+    T c = __shfl_up_sync(full, t[V - 1], 1);
+    if (sizeof(T) == 8) c = fma(rp[V - 1], __shfl_up_sync(full, t[V - 1], 2), c);
+#pragma unroll
+    for (int i = 0; i < V; ++i) t[i] = fma(rp[i], c, t[i]);
+#pragma unroll
+    for (int i = V - 2; i >= 0; --i) t[i] = fma(r, t[i + 1], t[i]);
+    c = __shfl_down_sync(full, t[0], 1);
+    if (sizeof(T) == 8) c = fma(rp[V - 1], __shfl_down_sync(full, t[0], 2), c);
+#pragma unroll
+    for (int i = 0; i < V; ++i) x[i] = fma(r, fma(rp[V - 1 - i], c, t[i]), x[i]);
+}
+
 // One residual sub-step for V cells m0..m0+V-1.  z[0..V+3] holds Q at cells
 // m0-2..m0+V+1, v[0..V] the interface velocities at m0..m0+V (interface k is the
 // left node of cell m0+k).  The flux through interface k (Eq. 6 with the PLM

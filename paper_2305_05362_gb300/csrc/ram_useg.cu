@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(256, V * sizeof(T) <= 32 ? 3 : 2)
 // residual sub-steps with shuffled neighbours, and the store of the segment's
 // interior [H4, H4 + stride) (whole vectors; the cells past N belong to no
 // segment).  Shared by the register-prefetch and shared-memory-ring kernels.
-template <int ORDER, int V, bool LIM, bool VL>
+template <int ORDER, int V, bool LIM, bool VL, bool A4 = false>
 __device__ __forceinline__ void seg_compute_f32(const RowParams<float> &P, int N, int nsub,
                                                 int H4, int stride, int off, bool use_dv,
                                                 int seg, int lane,
@@ -297,10 +297,12 @@ __device__ __forceinline__ void seg_compute_f32(const RowParams<float> &P, int N
         break;
     }
     float cur[V];
+    if constexpr (A4) a4_average(q);
     if constexpr (ORDER == 3)
         remap_warp3<V>(q, P, LIM, cur);
     else
         remap_group<float, ORDER, V>(q, P, LIM, cur);
+    if constexpr (A4) a4_points(cur);
     if (use_dv) {
         float v[V];
 #pragma unroll
@@ -443,7 +445,13 @@ struct RingLayout {
 // (shift_params_two_float), so no parameter kernel runs before it when every row
 // of the step takes this kernel; the phase is then advanced here too
 // (a.row_phase).  FP32 rows of at least 32 V + 12 cells.
-template <int ORDER, int V, bool LIM, bool VL>
+//
+// A4 (RAM_A4 plans): the cells are point values.  The window's averages are formed in
+// registers before the remap and the point values recovered after it (a4_average,
+// a4_points), with a wider halo: one launch and 12 bytes a cell, against four kernels
+// that passed the field through memory between them (512 x 4096 cells with a
+// residual, steps back to back: 45.4 and 9.9 us).
+template <int ORDER, int V, bool LIM, bool VL, bool A4>
 __global__ void __launch_bounds__(256, 3)
     k_useg_ring(StepArgs a, const int32_t *row_ids)
 {
@@ -471,8 +479,9 @@ __global__ void __launch_bounds__(256, 3)
     // halo at the ends of a warp's 32 V cells, whole vectors: the residual
     // sub-steps spoil nsub (donor) or 2 nsub (van Leer) cells at each end, and
     // the PPM remap with shared neighbours (remap_warp3) 1 more on the left and 2
-    // on the right; H4 cells on the left, HR on the right are not stored
-    const int spoil = nsub * (VL ? 2 : 1);
+    // on the right (and the averages' inverse kA4Halo at each end); H4 cells on the
+    // left, HR on the right are not stored
+    const int spoil = nsub * (VL ? 2 : 1) + (A4 ? kA4Halo<float> : 0);
     const int H4 = ((spoil + (ORDER == 3 ? 1 : 0) + VEC - 1) / VEC) * VEC;
     const int HR = ((spoil + (ORDER == 3 ? 2 : 0) + VEC - 1) / VEC) * VEC;
     const int stride = 32 * V - H4 - HR;
@@ -557,8 +566,8 @@ __global__ void __launch_bounds__(256, 3)
         // every lane has read the stage: refill it with the warp's next segment
         __syncwarp();
         issue(i + L::S);
-        seg_compute_f32<ORDER, V, LIM, VL>(P, N, nsub, H4, stride, off, use_dv, seg, lane, xw,
-                                           xv, qout, cmax);
+        seg_compute_f32<ORDER, V, LIM, VL, A4>(P, N, nsub, H4, stride, off, use_dv, seg, lane, xw,
+                                               xv, qout, cmax);
     }
     cp_async_wait<0>();
     if (cmax > 1.0f) atomicOr(a.err, ERR_CFL);
@@ -594,7 +603,9 @@ __device__ __noinline__ void seg_step_f64_any(const StepArgs &a, const RowParams
 }
 
 // One segment of k_useg_f64: output cells [out0, out0 + stride) of a row, 8 a lane.
-template <int ORDER, bool LIM, bool VL>
+// A4: point values, as in the ring kernel; out-of-the-ordinary windows (see above) keep
+// this form there, with their limiters decided in floating point.
+template <int ORDER, bool LIM, bool VL, bool A4>
 __device__ __forceinline__ void seg_f64(const StepArgs &a, const RowParams<double> &P, bool has_dv,
                                         int out0, int stride, int HL, int lane)
 {
@@ -632,7 +643,8 @@ __device__ __forceinline__ void seg_f64(const StepArgs &a, const RowParams<doubl
 #pragma unroll
     for (int k = 0; k < NW; ++k) top = max(top, mag_hi(w[k]));
     top = __reduce_max_sync(full, top);
-    if (__any_sync(full, other) || top >= kMagBig || (top < kMagSmall && top > 0)) {
+    const bool odd = __any_sync(full, other) || top >= kMagBig || (top < kMagSmall && top > 0);
+    if (!A4 && odd) {
         double cm = 0.0;
         seg_step_f64_any<ORDER, LIM, VL>(a, P, out0, end, lane, &cm);
         if (cm > 1.0) atomicOr(a.err, ERR_CFL);
@@ -642,6 +654,7 @@ __device__ __forceinline__ void seg_f64(const StepArgs &a, const RowParams<doubl
     double q[V + 4];
 #pragma unroll
     for (int j = 0; j < V + 4; ++j) q[j] = off ? w[j + 1] : w[j];
+    if (A4) a4_average(q);
     double cur[V];
     if (P.whole) {
 #pragma unroll
@@ -656,9 +669,14 @@ __device__ __forceinline__ void seg_f64(const StepArgs &a, const RowParams<doubl
 #pragma unroll
             for (int j = 0; j < V; ++j) {
                 const double D = dif[j] + dif[j + 1];
-                Dq[j + 1] = LIM ? mag_signed(mag_min(mag(D), mag_up(mag_min(mag(dif[j]), mag(dif[j + 1])), 2)),
-                                             dif[j], dif[j + 1])
-                                : D;
+                if (!LIM)
+                    Dq[j + 1] = D;
+                else if (A4 && odd)
+                    Dq[j + 1] = 2.0 * lim_dq(dif[j], dif[j + 1], true);
+                else
+                    Dq[j + 1] = mag_signed(
+                        mag_min(mag(D), mag_up(mag_min(mag(dif[j]), mag(dif[j + 1])), 2)), dif[j],
+                        dif[j + 1]);
             }
             Dq[0] = __shfl_up_sync(full, Dq[V], 1);
             Dq[V + 1] = __shfl_down_sync(full, Dq[1], 1);
@@ -669,7 +687,14 @@ __device__ __forceinline__ void seg_f64(const StepArgs &a, const RowParams<doubl
                 const double Er = Dq[j + 2] - Dq[j + 1];
                 double fa = fma(Er, -1.0 / 12.0, half_of(dif[j + 1]));
                 double fb = fma(El, 1.0 / 12.0, half_of(dif[j]));
-                if (LIM) {
+                if (LIM && A4 && odd) {
+                    if (fa * fb <= 0.0)
+                        fa = fb = 0.0;
+                    else if (fabs(fb) > 2.0 * fabs(fa))
+                        fb = 2.0 * fa;
+                    else if (fabs(fa) > 2.0 * fabs(fb))
+                        fa = 2.0 * fb;
+                } else if (LIM) {
                     const unsigned long long ma = mag(fa), mb = mag(fb);
                     const double a1 = mag_signed(mag_min(ma, mag_up(mb, 1)), fa, fb);
                     fb = mag_signed(mag_min(mb, mag_up(ma, 1)), fb, fa);
@@ -699,6 +724,7 @@ __device__ __forceinline__ void seg_f64(const StepArgs &a, const RowParams<doubl
 #pragma unroll
         for (int k = 0; k < V; ++k) cur[k] = (q[k + 2] - A[k]) + A[k + 1];
     }
+    if (A4) a4_points(cur);
     // ---- residual sub-steps (residual_group_cs's flux, each formed once) ----
     if (has_dv) {
         double wc[V];  // the swept part's midpoint: +-1 - c
@@ -719,7 +745,7 @@ __device__ __forceinline__ void seg_f64(const StepArgs &a, const RowParams<doubl
 #pragma unroll
                 for (int i = 0; i < V; ++i) {
                     const double dr = (i < V - 1 ? cur[i + 1] : zr) - cur[i];
-                    h[i] = half_vl_bits(dl, dr);
+                    h[i] = A4 && odd ? half_vl(dl, dr) : half_vl_bits(dl, dr);
                     dl = dr;
                 }
                 const double hl = __shfl_up_sync(full, h[V - 1], 1);
@@ -753,7 +779,7 @@ __device__ __forceinline__ void seg_f64(const StepArgs &a, const RowParams<doubl
 // kernel.  Few warps keep the FP64 pipe busy, so registers are plentiful; a segment a
 // warp (not a row a CTA) spreads rows of unequal sub-step counts over the SMs.
 // Bound by the FP64 pipe.
-template <int ORDER, bool LIM, bool VL>
+template <int ORDER, bool LIM, bool VL, bool A4>
 __global__ void __launch_bounds__(128, 3)
     k_useg_f64(StepArgs a, const int32_t *row_ids, const RowParams<double> *pars)
 {
@@ -766,13 +792,13 @@ __global__ void __launch_bounds__(128, 3)
     const bool has_dv = (a.mode != MODE_SHIFT) && (a.dv != nullptr) && nsub > 0;
     // halo, whole vectors: the sub-steps spoil nsub (donor) or 2 nsub cells at each end,
     // the remap with shared neighbours one on the right, the PPM one one more on each side
-    const int spoil = nsub * (VL ? 2 : 1);
+    const int spoil = nsub * (VL ? 2 : 1) + (A4 ? kA4Halo<double> : 0);
     const int HL = (spoil + (ORDER == 3 ? 1 : 0) + 1) / 2 * 2;
     const int HR = (spoil + (ORDER == 3 ? 2 : 1) + 1) / 2 * 2;
     const int stride = 32 * V - HL - HR;
     // one segment a warp, unless the row has more than a grid can
     for (int64_t seg = blockIdx.y * 4 + warp; seg * stride < N; seg += (int64_t)gridDim.y * 4)
-        seg_f64<ORDER, LIM, VL>(a, P, has_dv, (int)(seg * stride), stride, HL, lane);
+        seg_f64<ORDER, LIM, VL, A4>(a, P, has_dv, (int)(seg * stride), stride, HL, lane);
 }
 
 template <typename T, int ORDER, int V>
@@ -805,7 +831,7 @@ cudaError_t launch_useg_pf(const StepArgs &a, cudaStream_t s, int threads, const
     return launch_pdl(k_useg_pf<ORDER, false, false>, n_rows, threads, 0, s, a, row_ids, par);
 }
 
-template <int ORDER, int V, bool LIM, bool VL>
+template <int ORDER, int V, bool LIM, bool VL, bool A4>
 cudaError_t launch_ring_k(const Plan &p, const StepArgs &a, cudaStream_t s, int threads,
                           const int32_t *row_ids, int n_rows)
 {
@@ -814,40 +840,59 @@ cudaError_t launch_ring_k(const Plan &p, const StepArgs &a, cudaStream_t s, int 
     const int dev = p.device < 64 ? p.device : 63;
     if (!configured[dev]) {
         // the most any launch asks for (8 warps); the kernel's static arrays come on top
-        cudaError_t e = cudaFuncSetAttribute(k_useg_ring<ORDER, V, LIM, VL>,
+        cudaError_t e = cudaFuncSetAttribute(k_useg_ring<ORDER, V, LIM, VL, A4>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              8 * RingLayout<V>::warp_bytes);
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
-    return launch_pdl(k_useg_ring<ORDER, V, LIM, VL>, n_rows, threads, smem, s, a, row_ids);
+    return launch_pdl(k_useg_ring<ORDER, V, LIM, VL, A4>, n_rows, threads, smem, s, a, row_ids);
+}
+
+template <int ORDER, int V, bool A4>
+cudaError_t launch_ring_f(const Plan &p, const StepArgs &a, cudaStream_t s, int threads,
+                          const int32_t *row_ids, int n_rows)
+{
+    const bool lim = a.limiter != 0, vl = a.scheme == RAM_VANLEER;
+    if (lim && vl) return launch_ring_k<ORDER, V, true, true, A4>(p, a, s, threads, row_ids, n_rows);
+    if (lim) return launch_ring_k<ORDER, V, true, false, A4>(p, a, s, threads, row_ids, n_rows);
+    if (vl) return launch_ring_k<ORDER, V, false, true, A4>(p, a, s, threads, row_ids, n_rows);
+    return launch_ring_k<ORDER, V, false, false, A4>(p, a, s, threads, row_ids, n_rows);
 }
 
 template <int ORDER, int V>
 cudaError_t launch_useg_ring(const Plan &p, const StepArgs &a, cudaStream_t s, int threads,
                              const int32_t *row_ids, int n_rows)
 {
-    const bool lim = a.limiter != 0, vl = a.scheme == RAM_VANLEER;
-    if (lim && vl) return launch_ring_k<ORDER, V, true, true>(p, a, s, threads, row_ids, n_rows);
-    if (lim) return launch_ring_k<ORDER, V, true, false>(p, a, s, threads, row_ids, n_rows);
-    if (vl) return launch_ring_k<ORDER, V, false, true>(p, a, s, threads, row_ids, n_rows);
-    return launch_ring_k<ORDER, V, false, false>(p, a, s, threads, row_ids, n_rows);
+    if constexpr (ORDER == 3)
+        if (a.a4) return launch_ring_f<ORDER, V, true>(p, a, s, threads, row_ids, n_rows);
+    return launch_ring_f<ORDER, V, false>(p, a, s, threads, row_ids, n_rows);
 }
 
 // `longest`: cells of the longest row.
+template <int ORDER, bool A4>
+cudaError_t launch_f64_f(const StepArgs &a, cudaStream_t s, const int32_t *row_ids, int n_rows,
+                         int longest, const RowParams<double> *par)
+{
+    const bool lim = a.limiter != 0, vl = a.scheme == RAM_VANLEER;
+    // segments at the widest halo; the warps past a row's end leave
+    const int most = (a.mode != MODE_SHIFT && a.dv != nullptr ? RAM_MAX_NSUB * (vl ? 2 : 1) : 0) +
+                     (A4 ? kA4Halo<double> : 0);
+    const int stride = 256 - (most + 2) / 2 * 2 - (most + 3) / 2 * 2;
+    const dim3 grid(n_rows, std::min(((longest + stride - 1) / stride + 3) / 4, 65535));
+    void (*kern)(StepArgs, const int32_t *, const RowParams<double> *) =
+        lim ? (vl ? k_useg_f64<ORDER, true, true, A4> : k_useg_f64<ORDER, true, false, A4>)
+            : (vl ? k_useg_f64<ORDER, false, true, A4> : k_useg_f64<ORDER, false, false, A4>);
+    return launch_pdl(kern, grid, dim3(128), 0, s, a, row_ids, par);
+}
+
 template <int ORDER>
 cudaError_t launch_useg_f64(const StepArgs &a, cudaStream_t s, const int32_t *row_ids, int n_rows,
                             int longest, const RowParams<double> *par)
 {
-    const bool lim = a.limiter != 0, vl = a.scheme == RAM_VANLEER;
-    // segments at the widest halo; the warps past a row's end leave
-    const int most = a.mode != MODE_SHIFT && a.dv != nullptr ? RAM_MAX_NSUB * (vl ? 2 : 1) : 0;
-    const int stride = 256 - (most + 2) / 2 * 2 - (most + 3) / 2 * 2;
-    const dim3 grid(n_rows, std::min(((longest + stride - 1) / stride + 3) / 4, 65535));
-    void (*kern)(StepArgs, const int32_t *, const RowParams<double> *) =
-        lim ? (vl ? k_useg_f64<ORDER, true, true> : k_useg_f64<ORDER, true, false>)
-            : (vl ? k_useg_f64<ORDER, false, true> : k_useg_f64<ORDER, false, false>);
-    return launch_pdl(kern, grid, dim3(128), 0, s, a, row_ids, par);
+    if constexpr (ORDER == 3)
+        if (a.a4) return launch_f64_f<ORDER, true>(a, s, row_ids, n_rows, longest, par);
+    return launch_f64_f<ORDER, false>(a, s, row_ids, n_rows, longest, par);
 }
 
 template <int ORDER>
