@@ -51,8 +51,9 @@
 //
 // Measured against the per-order kernels (k_params with k_gwarp, or k_general with a
 // residual), us per step: 512 rows of 64 to 65536 cells (5.3 M cells), no limiter,
-// 111.4 / 52.0, with a van Leer residual 203.4 / 68.2; 1000 rows (9.5 M) limited
-// 196.0 / 94.5; one row of 4096 cells with a residual 14.3 / 8.7.  Tried: seven cells
+// 111.4 / 49.6, with a van Leer residual 203.4 / 66.0; 1000 rows (9.5 M) limited
+// 196.0 / 87.8; one row of 4096 cells with a residual 14.3 / 7.7.  Tried (when the batch
+// took 52.0): seven cells
 // per lane 57.5 (512 rows), seven or five CTAs per SM instead of six 52.9 and 52.9, the
 // lane's edges by side-by-side halvings instead of the walk 54.7, a loop without the
 // two predicated steps 54.9, the next node's position kept across edges 55.6.
@@ -202,11 +203,12 @@ struct Item {
     uint64_t S;                // the row's shift, fraction of the period in units of 2^-64
     int32_t row, n, start, count;
     int32_t most;              // most cells of a segment with its halo
-    int32_t order, qs;
+    int32_t order;
     int32_t p;                 // source cell of the first edge (halo included)
     int32_t nsub;
     float cf;                  // sub-step length
     float scale;               // position units -> the widths' units, about mean widths
+    uint32_t S32, period;      // shift and period in position units (mod 2^32)
 };
 
 struct SegCtx {
@@ -269,8 +271,10 @@ __device__ __forceinline__ void window_cells(const float (&q)[kV + 4], const flo
     reconstruct<ORDER, LIM>(q, h, c);
 #pragma unroll
     for (int i = 0; i < kV; ++i) {
+        const float m = q[i + 2] * h[i + 2];
+        if (ORDER < 4) c[i].w = m;
         sC[b + i] = c[i];
-        sM[b + i] = q[i + 2] * h[i + 2];
+        sM[b + i] = m;
     }
 }
 
@@ -365,8 +369,7 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
         float G[kV + 1], mass[kV];
         int w = kHR;
         uint32_t rw = 0;  // position of node w
-        // (edges of the windows before stay at the window's first node)
-        uint32_t ry = b < from ? 0u : min(xo[0] - off, kPast - 1u);
+        uint32_t ry = min(xo[0] - off, kPast - 1u);
         // the last node at or left of the edge: the nodes past the window are kPast,
         // so no bound is needed
 #pragma unroll
@@ -383,22 +386,29 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
             we[i] = w;
             de[i] = d;
             const float x = (float)d * g.scale;
-            const float4 c = sC[w];
-            G[i] = x * fmaf(x, fmaf(x, fmaf(x, c.w, c.z), c.y), c.x);
-            ry = b + i + 1 < from ? 0u : min(xo[i + 1] - off, kPast - 1u);
+            float4 c = sC[w];
+            if (order == 4) {
+                c.z = fmaf(x, c.w, c.z);
+                c.w = sM[w];
+            }
+            G[i] = x * fmaf(x, fmaf(x, c.z, c.y), c.x);
+            ry = min(xo[i + 1] - off, kPast - 1u);
+            // mostly no, one or two nodes: the first one's cell is the edge's own
             float m = 0.f;
-            // mostly no, one or two nodes
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const uint32_t r = sR[w + 1];
-                if (r <= ry) {
-                    m += sM[w];
-                    ++w;
-                    rw = r;
-                }
+            uint32_t r = sR[w + 1];
+            if (r <= ry) {
+                m = c.w;
+                ++w;
+                rw = r;
+            }
+            r = sR[w + 1];
+            if (r <= ry) {
+                m += sM[w];
+                ++w;
+                rw = r;
             }
             while (true) {
-                const uint32_t r = sR[w + 1];
+                r = sR[w + 1];
                 if (r > ry) break;
                 m += sM[w];
                 ++w;
@@ -419,21 +429,28 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
                 if (in) last = max(last, kV * (31 - __clz((int)in)) + i);
             }
         }
+        uint32_t least = de[0];
+#pragma unroll
+        for (int i = 1; i <= kV; ++i) least = min(least, de[i]);
 #pragma unroll
         for (int i = 0; i < kV; ++i) {
             const int j = b + i;
-            if (j >= from && j < last) {
-                // Eq. 18: the start of the right source cell less that of the left one,
-                // plus the cells passed from the left one on; Eq. 26
-                float val = (mass[i] + (G[i + 1] - G[i])) *
-                            rcp_approx((float)(xo[i + 1] - xo[i]) * g.scale);
-                if ((de[i] | de[i + 1]) == 0 && (i + 1 < kV ? we[i + 1] : w) == we[i] + 1) {
-                    // exactly one source cell: its value unchanged
+            // Eq. 18: the start of the right source cell less that of the left one, plus
+            // the cells passed from the left one on; Eq. 26
+            if (j >= from && j < last)
+                sP[j] = (mass[i] + (G[i + 1] - G[i])) *
+                        rcp_approx((float)(xo[i + 1] - xo[i]) * g.scale);
+        }
+        if (least == 0) {
+            // an edge on a node: a cell whose edges both are, on those of one source cell,
+            // takes its value unchanged
+#pragma unroll
+            for (int i = 0; i < kV; ++i)
+                if (b + i >= from && b + i < last && (de[i] | de[i + 1]) == 0 &&
+                    (i + 1 < kV ? we[i + 1] : w) == we[i] + 1) {
                     const int c = p + we[i] - kHR;
-                    val = g.qin[c < N ? c : c % N];
+                    sP[b + i] = g.qin[c < N ? c : c % N];
                 }
-                sP[j] = val;
-            }
         }
         __syncwarp();
         if (last >= ne) break;
@@ -453,6 +470,10 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
         off += sR[wl];
         p = (p + wl - kHR) % N;
         from = last;
+        // the edges before it are done: at the new window's first node
+#pragma unroll
+        for (int i = 0; i <= kV; ++i)
+            if (b + i < from) xo[i] = off;
         first = false;
         const int cb = p >= kHR ? p - kHR : p - kHR + N;
         cp_async_wait<0>();
@@ -580,10 +601,12 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
         it.count = t.count;
         it.most = t.window;
         it.order = row.order;
-        it.qs = qs;
         it.p = locate_cell(X, row.n, a.buckets + row.bucket_off, row.bucket_bits, a.density,
                            row.density, xe - S);
         it.S = S;
+        it.S32 = (uint32_t)((S + (qs > 0 ? 1ull << (qs - 1) : 0ull)) >> qs);
+        if (qs > 32) it.S32 &= (1u << (64 - qs)) - 1u;
+        it.period = qs > 32 ? 1u << (64 - qs) : 0u;
         it.nsub = P.nsub;
         it.cf = P.cf;
         // a power of two, so that widths and offsets round once; a mean cell is in [1, 2)
@@ -633,7 +656,7 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
         e = e < 0 ? e + N : e;
         const int cb = nx_p >= kHR ? nx_p - kHR : nx_p - kHR + N;
         const uint32_t *X32 = a.x32 + it.mesh_off;
-        const uint32_t period = it.qs > 32 ? 1u << (64 - it.qs) : 0u;
+        const uint32_t period = it.period;
         copy_cells(smem_u32(w32 + kOffQ + 2), static_cast<const float *>(a.q_in) + it.cell_off, cb, N,
                    lane);
         copy_nodes(w32 + kOffX + 2, X32, cb, N, period, lane);
@@ -644,7 +667,6 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
     cp_async_commit();
     while (nx < n_it) {
         const Item &it = s_item[nx];
-        const int qs = it.qs;
         SegCtx g;
         g.X32 = a.x32 + it.mesh_off;
         g.qin = static_cast<const float *>(a.q_in) + it.cell_off;
@@ -659,9 +681,8 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
         g.vl = R == 2;
         g.scale = it.scale;
         g.cf = it.cf;
-        g.S32 = (uint32_t)((it.S + (qs > 0 ? 1ull << (qs - 1) : 0ull)) >> qs);
-        if (qs > 32) g.S32 &= (1u << (64 - qs)) - 1u;
-        g.period = qs > 32 ? 1u << (64 - qs) : 0u;
+        g.S32 = it.S32;
+        g.period = it.period;
         g.err = a.err;
         const int i0 = it.start + nx_piece * nx_seg;
         const int cnt = min(nx_seg, it.start + it.count - i0);
