@@ -343,7 +343,9 @@ __global__ void __launch_bounds__(512)
 
     // The first general launch of a step waits for the parameter kernel; the
     // later ones are launched once it has (each launch lets the next start as
-    // soon as its own wait is over) and touch other rows, so they run alongside.
+    // soon as its own wait is over) and touch other rows, so they run alongside and
+    // wait for the one before only at their end (a kernel that waits for the last of
+    // them waits for all).
     if (wait) pdl_wait();
     pdl_trigger();
     const RowParams<T> P = pars[tile.row];
@@ -395,7 +397,10 @@ __global__ void __launch_bounds__(512)
     if (nsub > 0)
         for (int j = tid; j <= nq; j += nth) sV[j] = dvp[wrap_index((int64_t)tile.start - H + j, N)];
     __syncthreads();
-    if (s_bad) return;
+    if (s_bad) {
+        if (!wait) pdl_wait();
+        return;
+    }
     const int plo = s_plo, W = s_W;
     const uint64_t xbase = s_xbase;
     const int wb = wrap_index((int64_t)plo - kHR, N);  // cell of slot 0
@@ -511,6 +516,7 @@ __global__ void __launch_bounds__(512)
         __syncthreads();
     }
     for (int i = tid; i < T_out; i += nth) qout[tile.start + i] = cur[H + i];
+    if (!wait) pdl_wait();
 }
 
 // The shift step alone (no residual) on non-uniform rows, without shared
@@ -625,6 +631,7 @@ __global__ void __launch_bounds__(512)
             qout[g] = val;
         }
     }
+    if (!wait) pdl_wait();
 }
 
 // A list of non-uniform tiles of one order for the general kernels: the rows that the

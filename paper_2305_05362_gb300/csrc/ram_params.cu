@@ -12,7 +12,9 @@ namespace {
 template <typename T>
 __global__ void __launch_bounds__(32) k_params(StepArgs a, int n_rows, RowParams<T> *out)
 {
-    // the row kernels that follow may start now; they wait for these results
+    // the previous kernel may still be reading the parameters of its launch; once it has
+    // finished, the row kernels that follow may start (they wait for these results)
+    pdl_wait();
     pdl_trigger();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n_rows) return;
@@ -29,12 +31,10 @@ cudaError_t launch_params(const Plan &p, ram_dtype dt, const StepArgs &a, cudaSt
     const int threads = 32;
     const int blocks = (p.n_rows + threads - 1) / threads;
     if (dt == RAM_F32)
-        k_params<float><<<blocks, threads, 0, s>>>(a, p.n_rows,
-                                                   static_cast<RowParams<float> *>(p.row_par));
-    else
-        k_params<double><<<blocks, threads, 0, s>>>(a, p.n_rows,
-                                                    static_cast<RowParams<double> *>(p.row_par));
-    return cudaGetLastError();
+        return launch_pdl(k_params<float>, blocks, threads, 0, s, a, p.n_rows,
+                          static_cast<RowParams<float> *>(p.row_par));
+    return launch_pdl(k_params<double>, blocks, threads, 0, s, a, p.n_rows,
+                      static_cast<RowParams<double> *>(p.row_par));
 }
 
 }  // namespace ram
