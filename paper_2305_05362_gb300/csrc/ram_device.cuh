@@ -39,6 +39,13 @@ __device__ __forceinline__ float minxs(float a, float b)
     asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
     return d;
 }
+// max(|a|, |b|, |c|)
+__device__ __forceinline__ float max_abs3(float a, float b, float c)
+{
+    float d;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
 __device__ __forceinline__ double minxs(double a, double b)
 {
     const double m = fmin(fabs(a), fabs(b));

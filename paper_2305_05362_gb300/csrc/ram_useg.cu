@@ -312,13 +312,10 @@ __device__ __forceinline__ void seg_compute_f32(const RowParams<float> &P, int N
             v[4 * c + 2] = xv[c].z;
             v[4 * c + 3] = xv[c].w;
         }
-        float cm = 0.0f;
 #pragma unroll
-        for (int k = 0; k < V; ++k) {
-            v[k] *= P.cf;  // the faces' Courant numbers, the same in every sub-step
-            cm = fmaxf(cm, fabsf(v[k]));
-        }
-        cmax = fmaxf(cmax, cm);
+        for (int k = 0; k < V; ++k) v[k] *= P.cf;  // the faces' Courant numbers
+#pragma unroll
+        for (int k = 0; k < V; k += 2) cmax = max_abs3(cmax, v[k], v[k + 1]);
         for (int sub = 0; sub < nsub; ++sub) residual_warp<V, VL>(cur, v);
     }
     const int li0 = lane * V;
