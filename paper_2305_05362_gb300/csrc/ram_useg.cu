@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cstdint>
 #include <type_traits>
 
@@ -257,18 +258,28 @@ __global__ void __launch_bounds__(256, V * sizeof(T) <= 32 ? 3 : 2)
 // remap of the lane's V cells (its source cells start at w[off + 2]), the
 // residual sub-steps with shuffled neighbours, and the store of the segment's
 // interior [H4, H4 + stride) (whole vectors; the cells past N belong to no
-// segment).  Shared by the register-prefetch and shared-memory-ring kernels.
+// segment).  m0: the lane's first cell; store_end: per vector of the lane, N inside
+// that interior (store_ends).  Shared by the register-prefetch and
+// shared-memory-ring kernels.
+template <int V>
+__device__ __forceinline__ void store_ends(int N, int H4, int stride, int lane, int (&end)[V / 4])
+{
+#pragma unroll
+    for (int c = 0; c < V / 4; ++c) {
+        const int li = lane * V + 4 * c;
+        end[c] = li >= H4 && li < H4 + stride ? N : INT_MIN;
+    }
+}
+
 template <int ORDER, int V, bool LIM, bool VL, bool A4 = false>
-__device__ __forceinline__ void seg_compute_f32(const RowParams<float> &P, int N, int nsub,
-                                                int H4, int stride, int off, bool use_dv,
-                                                int seg, int lane,
+__device__ __forceinline__ void seg_compute_f32(const RowParams<float> &P, int nsub, int m0,
+                                                int off, bool use_dv,
+                                                const int (&store_end)[V / 4],
                                                 const float4 (&xw)[(V + 12) / 4],
                                                 const float4 (&xv)[V / 4], float *qout,
                                                 float &cmax)
 {
     constexpr int VEC = 4, NW = V + 12;
-    const int out0 = seg * stride;
-    const int m0 = out0 - H4 + lane * V;
     float w[NW];
 #pragma unroll
     for (int c = 0; c < NW / VEC; ++c) {
@@ -318,14 +329,11 @@ __device__ __forceinline__ void seg_compute_f32(const RowParams<float> &P, int N
         for (int k = 0; k < V; k += 2) cmax = max_abs3(cmax, v[k], v[k + 1]);
         for (int sub = 0; sub < nsub; ++sub) residual_warp<V, VL>(cur, v);
     }
-    const int li0 = lane * V;
 #pragma unroll
-    for (int c = 0; c < V / VEC; ++c) {
-        const int li = li0 + c * VEC;
-        if (li >= H4 && li < H4 + stride && m0 + c * VEC < N)
+    for (int c = 0; c < V / VEC; ++c)
+        if (m0 + c * VEC < store_end[c])
             *reinterpret_cast<float4 *>(qout + m0 + c * VEC) =
                 make_float4(cur[4 * c], cur[4 * c + 1], cur[4 * c + 2], cur[4 * c + 3]);
-    }
 }
 
 // The same step with the loads of a warp's next segment in flight while it
@@ -359,6 +367,9 @@ __global__ void __launch_bounds__(256, 2)
     const int off = ((-P.K - 1) % VEC + VEC) % VEC;
     const bool use_dv = has_dv && nsub > 0;
     float cmax = 0.0f;
+
+    int store_end[V / 4];
+    store_ends<V>(N, H4, stride, lane, store_end);
 
     struct Raw {
         float4 w[NW / VEC];
@@ -396,8 +407,8 @@ __global__ void __launch_bounds__(256, 2)
         }
     };
     auto compute = [&](int seg, const Raw &x) {
-        seg_compute_f32<ORDER, V, LIM, VL>(P, N, nsub, H4, stride, off, use_dv, seg, lane, x.w,
-                                           x.v, qout, cmax);
+        seg_compute_f32<ORDER, V, LIM, VL>(P, nsub, seg * stride - H4 + lane * V, off, use_dv,
+                                           store_end, x.w, x.v, qout, cmax);
     };
 
     Raw ra, rb;
@@ -411,6 +422,15 @@ __global__ void __launch_bounds__(256, 2)
         if (s1 < nseg) compute(s1, rb);
     }
     if (cmax > 1.0f) atomicOr(a.err, ERR_CFL);
+}
+
+// The row's next segment (one lane asks; as atomicAdd the compiler would gather the
+// lanes' requests first).
+__device__ __forceinline__ int counter_next(uint32_t counter)
+{
+    int v;
+    asm volatile("atom.shared.add.u32 %0, [%1], 1;" : "=r"(v) : "r"(counter) : "memory");
+    return v;
 }
 
 // Shared-memory layout of the ring kernel, per warp: S stages, each the warp
@@ -497,19 +517,24 @@ __global__ void __launch_bounds__(256, 3)
     // start.  Lane l copies the 16-byte chunks l, l + 32, ... of the window and
     // of the dv range.
     const uint32_t ring_s = smem_u32(ring) + 16u * lane;
+    const uint32_t seg_counter = smem_u32(&seg_next);
     constexpr uint32_t kStageBytes = L::stage_floats * 4;
-    const int wshift = P.K + 1 + off + VEC;  // window start = w0 - wshift
+    // the window of the segment at cell 0 starts at wstart, reduced to [0, N)
+    const int wstart = wrap2(-H4 - (P.K + 1 + off + VEC), N);
+    const int lane_m0 = lane * V - H4;
+    int store_end[V / 4];
+    store_ends<V>(N, H4, stride, lane, store_end);
     const float *const qlane = qin + 4 * lane;
     const float *const dlane = use_dv ? dvp + 4 * lane : nullptr;
     auto issue = [&](int i) {
         int seg = 0;
-        if (lane == 0) seg = atomicAdd(&seg_next, 1);
+        if (lane == 0) seg = counter_next(seg_counter);
         seg = __shfl_sync(0xffffffffu, seg, 0);
         slot[i % L::S] = seg;  // every lane writes the same value
         if (seg < nseg) {
-            const int w0 = seg * stride - H4;
+            const int o0 = seg * stride;  // < N
             const uint32_t sq = ring_s + (uint32_t)(i % L::S) * kStageBytes;
-            const int wb = wrap2(w0 - wshift, N);
+            const int wb = wrap1(wstart + o0, N);
             if (wb + L::WQ <= N) {
                 const float *src = qlane + wb;
 #pragma unroll
@@ -523,7 +548,7 @@ __global__ void __launch_bounds__(256, 3)
                 }
             }
             if (use_dv) {
-                const int wv = wrap2(w0, N);
+                const int wv = o0 < H4 ? o0 - H4 + N : o0 - H4;
                 const uint32_t sv = sq + L::WQ * 4;
                 if (wv + L::WV <= N) {
                     const float *src = dlane + wv;
@@ -563,8 +588,8 @@ __global__ void __launch_bounds__(256, 3)
         // every lane has read the stage: refill it with the warp's next segment
         __syncwarp();
         issue(i + L::S);
-        seg_compute_f32<ORDER, V, LIM, VL, A4>(P, N, nsub, H4, stride, off, use_dv, seg, lane, xw,
-                                               xv, qout, cmax);
+        seg_compute_f32<ORDER, V, LIM, VL, A4>(P, nsub, seg * stride + lane_m0, off, use_dv,
+                                               store_end, xw, xv, qout, cmax);
     }
     cp_async_wait<0>();
     if (cmax > 1.0f) atomicOr(a.err, ERR_CFL);
