@@ -223,11 +223,6 @@ struct SegCtx {
     int *err;
 };
 
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-
 // Values of cells first .. first + kWin - 1 (cyclic, first in [0, N)) to dst, 4 bytes a
 // lane and copy.
 __device__ __forceinline__ void copy_cells(uint32_t dst, const float *src, int first, int N,
@@ -236,10 +231,10 @@ __device__ __forceinline__ void copy_cells(uint32_t dst, const float *src, int f
     if (first + kWin <= N) {
         const float *s = src + first + lane;
 #pragma unroll
-        for (int i = 0; i < kV; ++i) cp_async4(dst + 4u * (lane + 32 * i), s + 32 * i);
+        for (int i = 0; i < kV; ++i) cp_async4_s(dst + 4u * (lane + 32 * i), s + 32 * i);
     } else {
 #pragma unroll 1
-        for (int k = lane; k < kWin; k += 32) cp_async4(dst + 4u * k, src + (first + k) % N);
+        for (int k = lane; k < kWin; k += 32) cp_async4_s(dst + 4u * k, src + (first + k) % N);
     }
 }
 
@@ -251,8 +246,8 @@ __device__ __forceinline__ void copy_nodes(uint32_t *dst, const uint32_t *src, i
         const uint32_t *s = src + first + lane;
         const uint32_t d = smem_u32(dst + lane);
 #pragma unroll
-        for (int i = 0; i < kV; ++i) cp_async4(d + 128u * i, s + 32 * i);
-        if (lane == 0) cp_async4(d + 4u * kWin, s + kWin);
+        for (int i = 0; i < kV; ++i) cp_async4_s(d + 128u * i, s + 32 * i);
+        if (lane == 0) cp_async4_s(d + 4u * kWin, s + kWin);
     } else {
 #pragma unroll 1
         for (int k = lane; k <= kWin; k += 32) {
@@ -313,8 +308,8 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
         for (int k = lane; k <= ne; k += 32) {
             int c = a0 + k;
             c = c >= N ? c - N : c;  // ne < N
-            cp_async4(d + 4u * k, g.dvp + c);
-            cp_async4(d + 4u * (kOffH - kOffV) + 4u * k, g.dx + c);
+            cp_async4_s(d + 4u * k, g.dvp + c);
+            cp_async4_s(d + 4u * (kOffH - kOffV) + 4u * k, g.dx + c);
         }
     }
     cp_async_commit();

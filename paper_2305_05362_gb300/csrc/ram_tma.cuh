@@ -82,6 +82,11 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 }
 
 // The same copy to a shared-memory address given as a 32-bit shared-window offset.
+__device__ __forceinline__ void cp_async4_s(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+
 __device__ __forceinline__ void cp_async16_s(uint32_t dst, const void *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");

@@ -254,13 +254,8 @@ __global__ void __launch_bounds__(256, V * sizeof(T) <= 32 ? 3 : 2)
     if (cmax > T(1)) atomicOr(a.err, ERR_CFL);
 }
 
-// One FP32 warp segment from its raw window and dv vectors (in registers): the
-// remap of the lane's V cells (its source cells start at w[off + 2]), the
-// residual sub-steps with shuffled neighbours, and the store of the segment's
-// interior [H4, H4 + stride) (whole vectors; the cells past N belong to no
-// segment).  m0: the lane's first cell; store_end: per vector of the lane, N inside
-// that interior (store_ends).  Shared by the register-prefetch and
-// shared-memory-ring kernels.
+// Per vector of the lane: N inside the segment's interior [H4, H4 + stride), which the
+// warp stores, else no cell.
 template <int V>
 __device__ __forceinline__ void store_ends(int N, int H4, int stride, int lane, int (&end)[V / 4])
 {
@@ -271,24 +266,20 @@ __device__ __forceinline__ void store_ends(int N, int H4, int stride, int lane, 
     }
 }
 
-template <int ORDER, int V, bool LIM, bool VL, bool A4 = false>
-__device__ __forceinline__ void seg_compute_f32(const RowParams<float> &P, int nsub, int m0,
-                                                int off, bool use_dv,
-                                                const int (&store_end)[V / 4],
-                                                const float4 (&xw)[(V + 12) / 4],
-                                                const float4 (&xv)[V / 4], float *qout,
-                                                float &cmax)
+// The lane's source cells q[0 .. V + 4] (p0 - 2 on) from its 16-byte aligned window, off
+// cells into it.
+template <int V>
+__device__ __forceinline__ void window_at(const float4 (&xw)[(V + 12) / 4], int off, float (&q)[V + 5])
 {
-    constexpr int VEC = 4, NW = V + 12;
+    constexpr int NW = V + 12;
     float w[NW];
 #pragma unroll
-    for (int c = 0; c < NW / VEC; ++c) {
+    for (int c = 0; c < NW / 4; ++c) {
         w[4 * c] = xw[c].x;
         w[4 * c + 1] = xw[c].y;
         w[4 * c + 2] = xw[c].z;
         w[4 * c + 3] = xw[c].w;
     }
-    float q[V + 5];
     switch (off) {
     case 0:
 #pragma unroll
@@ -307,6 +298,21 @@ __device__ __forceinline__ void seg_compute_f32(const RowParams<float> &P, int n
         for (int j = 0; j < V + 5; ++j) q[j] = w[j + 5];
         break;
     }
+}
+
+// One FP32 warp segment from its source cells q[0 .. V + 4] (p0 - 2 on) and raw dv
+// vectors, in registers: the remap of the lane's V cells, the residual sub-steps with
+// shuffled neighbours, and the store of the segment's interior (whole vectors; the
+// cells past N belong to no segment).  m0: the lane's first cell; store_end: see
+// store_ends.  Shared by the register-prefetch and shared-memory-ring kernels.
+template <int ORDER, int V, bool LIM, bool VL, bool A4 = false>
+__device__ __forceinline__ void seg_compute_f32(const RowParams<float> &P, int nsub, int m0,
+                                                bool use_dv, const int (&store_end)[V / 4],
+                                                float (&q)[V + 5],
+                                                const float4 (&xv)[V / 4], float *qout,
+                                                float &cmax)
+{
+    constexpr int VEC = 4;
     float cur[V];
     if constexpr (A4) a4_average(q);
     if constexpr (ORDER == 3)
@@ -407,8 +413,10 @@ __global__ void __launch_bounds__(256, 2)
         }
     };
     auto compute = [&](int seg, const Raw &x) {
-        seg_compute_f32<ORDER, V, LIM, VL>(P, nsub, seg * stride - H4 + lane * V, off, use_dv,
-                                           store_end, x.w, x.v, qout, cmax);
+        float q[V + 5];
+        window_at<V>(x.w, off, q);
+        seg_compute_f32<ORDER, V, LIM, VL>(P, nsub, seg * stride - H4 + lane * V, use_dv, store_end,
+                                           q, x.v, qout, cmax);
     };
 
     Raw ra, rb;
@@ -434,27 +442,31 @@ __device__ __forceinline__ int counter_next(uint32_t counter)
 }
 
 // Shared-memory layout of the ring kernel, per warp: S stages, each the warp
-// segment's source window (32 V + 12 cells from a 16-byte aligned start)
-// followed by its dv (32 V cells).  One stage: the warp reads it into registers
-// before computing, so the copies of its next segment already overlap the
+// segment's source window from source cell p0 - 2 on (32 V cells and the remap's
+// halo), followed by its dv (32 V cells).  One stage: the warp reads it into
+// registers before computing, so the copies of its next segment already overlap the
 // computation of the current one; more stages in flight made the step slower
 // (the segments a warp claims ahead are no longer handed out to the warps that
 // finish first: 15.4, 15.9, 17.0 and 18.1 µs per step for 1-4 stages on the
 // 1024 x 4096 disk).
-template <int V>
+template <int ORDER, int V>
 struct RingLayout {
-    static constexpr int WQ = 32 * V + 12;
+    static constexpr int NQ = ORDER == 4 ? V + 8 : V + 4;  // cells a lane reads
+    static constexpr int WQ = 31 * V + NQ;
     static constexpr int WV = 32 * V;
     static constexpr int S = 1;
     static constexpr int stage_floats = WQ + WV;
     static constexpr int warp_bytes = S * stage_floats * 4;
-    static_assert((stage_floats * 4) % 16 == 0, "16-byte aligned stages");
+    static_assert(WQ % 4 == 0 && (stage_floats * 4) % 16 == 0, "16-byte aligned stages");
 };
 
 // The same step with each warp's segments staged through a ring of S shared-memory
-// stages filled by asynchronous 16-byte copies (the data does not pass through
-// registers until the segment is computed), so that S segments per warp are in
-// flight.  A warp reads a stage into registers, refills it at once with the
+// stages filled by asynchronous copies (the data does not pass through registers
+// until the segment is computed), so that S segments per warp are in flight: 16 bytes
+// a lane for dv, 4 for the window, whose start the shift leaves on any word -- so that
+// every lane's cells lie at the same 16-byte boundary of the stage (with 16-byte copies
+// each lane read five vectors and moved its cells into place by the offset in them:
+// 15.2 us on the 1024 x 4096 disk and 312.9 on the 8192 x 16384 one, 14.8 and 305.2 so).  A warp reads a stage into registers, refills it at once with the
 // copies of its next segment and computes.  The warps of a row take its segments
 // from a counter in shared memory as they issue the copies, so a warp on a
 // crowded scheduler takes fewer of them and the row's CTA finishes with its
@@ -472,8 +484,8 @@ template <int ORDER, int V, bool LIM, bool VL, bool A4>
 __global__ void __launch_bounds__(256, 3)
     k_useg_ring(StepArgs a, const int32_t *row_ids)
 {
-    using L = RingLayout<V>;
-    constexpr int VEC = 4, NW = V + 12;
+    using L = RingLayout<ORDER, V>;
+    constexpr int VEC = 4;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int seg_next;                // the row's next segment to hand out
     __shared__ int seg_slot[8][L::S];       // segment held by each warp's stages
@@ -506,25 +518,24 @@ __global__ void __launch_bounds__(256, 3)
     const float *qin = static_cast<const float *>(a.q_in) + P.cell_off;
     const float *dvp = has_dv ? static_cast<const float *>(a.dv) + P.cell_off : nullptr;
     float *qout = static_cast<float *>(a.q_out) + P.cell_off;
-    const int off = ((-P.K - 1) % VEC + VEC) % VEC;
     const bool use_dv = has_dv && nsub > 0;
     __syncthreads();  // seg_next is set
 
     // copies of the segment this warp takes next into stage i % S, one commit
     // group per stage use (empty once the row's segments are all handed out, so
-    // that group i is always the (i+1)-th).  The window starts at the 16-byte
-    // aligned cell wb in [0, N); a vector past the row's end comes from its
-    // start.  Lane l copies the 16-byte chunks l, l + 32, ... of the window and
-    // of the dv range.
-    const uint32_t ring_s = smem_u32(ring) + 16u * lane;
+    // that group i is always the (i+1)-th).  The window starts at cell wb in [0, N);
+    // a cell (a vector of dv) past the row's end comes from its start.  Lane l copies
+    // the cells l, l + 32, ... of the window and the 16-byte chunks l, l + 32, ... of
+    // the dv range.
+    const uint32_t ring_s = smem_u32(ring);
     const uint32_t seg_counter = smem_u32(&seg_next);
     constexpr uint32_t kStageBytes = L::stage_floats * 4;
     // the window of the segment at cell 0 starts at wstart, reduced to [0, N)
-    const int wstart = wrap2(-H4 - (P.K + 1 + off + VEC), N);
+    const int wstart = wrap2(-H4 - (P.K + 3), N);
     const int lane_m0 = lane * V - H4;
     int store_end[V / 4];
     store_ends<V>(N, H4, stride, lane, store_end);
-    const float *const qlane = qin + 4 * lane;
+    const float *const qlane = qin + lane;
     const float *const dlane = use_dv ? dvp + 4 * lane : nullptr;
     auto issue = [&](int i) {
         int seg = 0;
@@ -535,21 +546,22 @@ __global__ void __launch_bounds__(256, 3)
             const int o0 = seg * stride;  // < N
             const uint32_t sq = ring_s + (uint32_t)(i % L::S) * kStageBytes;
             const int wb = wrap1(wstart + o0, N);
+            const uint32_t sl = sq + 4u * lane;
             if (wb + L::WQ <= N) {
                 const float *src = qlane + wb;
 #pragma unroll
-                for (int j = 0; j < (L::WQ / 4 + 31) / 32; ++j)
-                    if (lane + 32 * j < L::WQ / 4) cp_async16_s(sq + 512u * j, src + 128 * j);
+                for (int j = 0; j < (L::WQ + 31) / 32; ++j)
+                    if (32 * j + 32 <= L::WQ || lane < L::WQ - 32 * j)
+                        cp_async4_s(sl + 128u * j, src + 32 * j);
             } else {
 #pragma unroll
-                for (int j = 0; j < (L::WQ / 4 + 31) / 32; ++j) {
-                    const int c = lane + 32 * j;
-                    if (c < L::WQ / 4) cp_async16_s(sq + 512u * j, qin + wrap1(wb + 4 * c, N));
-                }
+                for (int j = 0; j < (L::WQ + 31) / 32; ++j)
+                    if (32 * j + 32 <= L::WQ || lane < L::WQ - 32 * j)
+                        cp_async4_s(sl + 128u * j, qin + wrap1(wb + lane + 32 * j, N));
             }
             if (use_dv) {
                 const int wv = o0 < H4 ? o0 - H4 + N : o0 - H4;
-                const uint32_t sv = sq + L::WQ * 4;
+                const uint32_t sv = sq + L::WQ * 4 + 16u * lane;
                 if (wv + L::WV <= N) {
                     const float *src = dlane + wv;
 #pragma unroll
@@ -578,9 +590,17 @@ __global__ void __launch_bounds__(256, 3)
         cp_async_wait<L::S - 1>();
         __syncwarp();
         const uint32_t sq = lds0 + (uint32_t)(i % L::S) * kStageBytes;
-        float4 xw[NW / VEC], xv[V / VEC];
+        float q[V + 5];
+        float4 xv[V / VEC];
 #pragma unroll
-        for (int c = 0; c < NW / VEC; ++c) xw[c] = lds128(sq + 16u * c);
+        for (int c = 0; c < L::NQ / VEC; ++c) {
+            const float4 x = lds128(sq + 16u * c);
+            const float e[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (4 * c + k < V + 5) q[4 * c + k] = e[k];
+        }
+        if (L::NQ < V + 5) q[V + 4] = 0.0f;  // read by order 4 only
         if (use_dv) {
 #pragma unroll
             for (int c = 0; c < V / VEC; ++c) xv[c] = lds128(sq + L::WQ * 4 + 16u * c);
@@ -588,8 +608,8 @@ __global__ void __launch_bounds__(256, 3)
         // every lane has read the stage: refill it with the warp's next segment
         __syncwarp();
         issue(i + L::S);
-        seg_compute_f32<ORDER, V, LIM, VL, A4>(P, nsub, seg * stride + lane_m0, off, use_dv,
-                                               store_end, xw, xv, qout, cmax);
+        seg_compute_f32<ORDER, V, LIM, VL, A4>(P, nsub, seg * stride + lane_m0, use_dv, store_end, q,
+                                               xv, qout, cmax);
     }
     cp_async_wait<0>();
     if (cmax > 1.0f) atomicOr(a.err, ERR_CFL);
@@ -857,14 +877,14 @@ template <int ORDER, int V, bool LIM, bool VL, bool A4>
 cudaError_t launch_ring_k(const Plan &p, const StepArgs &a, cudaStream_t s, int threads,
                           const int32_t *row_ids, int n_rows)
 {
-    const size_t smem = (size_t)(threads / 32) * RingLayout<V>::warp_bytes;
+    const size_t smem = (size_t)(threads / 32) * RingLayout<ORDER, V>::warp_bytes;
     static bool configured[64] = {false};
     const int dev = p.device < 64 ? p.device : 63;
     if (!configured[dev]) {
         // the most any launch asks for (8 warps); the kernel's static arrays come on top
         cudaError_t e = cudaFuncSetAttribute(k_useg_ring<ORDER, V, LIM, VL, A4>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             8 * RingLayout<V>::warp_bytes);
+                                             8 * RingLayout<ORDER, V>::warp_bytes);
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
