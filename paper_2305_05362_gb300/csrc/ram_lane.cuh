@@ -124,37 +124,33 @@ __device__ __forceinline__ void remap_warp3(const float (&q)[V + 5], const RowPa
         return;
     }
     const unsigned full = 0xffffffffu;
-    // in quarters of the differences (exact scalings): 2 dQ / 4 = minxs(D / 4, max(minxs(dif,
-    // dif'), 0)) spares the factor 4, and a / 2, b / 2 come from the same quarters
-    float dif[V + 1], qd[V + 1];  // dif[i] = Q(p0-1+i+1) - Q(p0-1+i), i = 0..V, and dif / 4
+    float dif[V + 1];  // dif[i] = Q(p0-1+i+1) - Q(p0-1+i), i = 0..V
 #pragma unroll
-    for (int i = 0; i <= V; ++i) {
-        dif[i] = q[i + 2] - q[i + 1];
-        qd[i] = 0.25f * dif[i];
-    }
-    float Dq[V + 2];   // 2 dQ / 4 of cells p0-1 .. p0+V; own cells at Dq[1..V]
+    for (int i = 0; i <= V; ++i) dif[i] = q[i + 2] - q[i + 1];
+    float Dq[V + 2];   // 2 dQ of cells p0-1 .. p0+V; own cells at Dq[1..V]
 #pragma unroll
     for (int j = 0; j < V; ++j) {
-        const float D = qd[j] + qd[j + 1];
-        Dq[j + 1] = lim ? minxs(D, fmaxf(minxs(dif[j], dif[j + 1]), 0.0f)) : D;
+        const float D = dif[j] + dif[j + 1];
+        Dq[j + 1] = lim ? minxs(D, fmaxf(4.0f * minxs(dif[j], dif[j + 1]), 0.0f)) : D;
     }
     Dq[0] = __shfl_up_sync(full, Dq[V], 1);
     Dq[V + 1] = __shfl_down_sync(full, Dq[1], 1);
     float E[V + 1];    // E[i] = Dq(p0+i) - Dq(p0+i-1)
 #pragma unroll
     for (int i = 0; i <= V; ++i) E[i] = Dq[i + 1] - Dq[i];
-    const float xi = P.c[3], cR = 2.0f * P.c[1], cL = 2.0f * P.c[0];
+    const float xi = P.c[3], cR = 0.5f * P.c[1], cL = 0.5f * P.c[0];
     float A[V + 1];
 #pragma unroll
     for (int j = 0; j < V; ++j) {
-        // cell p0+j: a / 2 (right face) and b / 2 (left face)
-        const float a = fmaf(E[j + 1], -1.0f / 6.0f, qd[j + 1]);
-        const float b = fmaf(E[j], 1.0f / 6.0f, qd[j]);
+        // cell p0+j: 2a (right face) and 2b (left face)
+        const float a = fmaf(E[j + 1], -1.0f / 6.0f, dif[j + 1]);
+        const float b = fmaf(E[j], 1.0f / 6.0f, dif[j]);
         float G;
         if (lim) {
-            const float u = fmaxf(minxs(a, b + b), 0.0f);  // |a'| / 2
-            const float v = fmaxf(minxs(b, a + a), 0.0f);  // |b'| / 2
-            G = xorsign(fmaf(cR, u, -cL * v), a);
+            // both bounds from g = min(|a|, |b|) (0 at an extremum): |a'| = min(|a|, 2|b|) =
+            // min(|a|, 2g), |b'| = min(|b|, 2|a|) = min(|b|, 2g)
+            const float g = fmaxf(minxs(a, b), 0.0f), g2 = g + g;
+            G = xorsign(fmaf(cR, fminf(fabsf(a), g2), -cL * fminf(fabsf(b), g2)), a);
         } else {
             G = fmaf(cR, a, -cL * b);
         }
