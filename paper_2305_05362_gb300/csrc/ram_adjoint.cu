@@ -125,6 +125,19 @@ __device__ __forceinline__ void load_cells(const T *row, int wfirst, int lane, i
     }
 }
 
+// Whether two-float arithmetic holds a row's shift as well as FP64 does for FP32 cells
+// (the fraction of a cell to 2^-26): less than 2^20 cells, the factors of v0 dt N / L zero
+// or well inside the FP32 range.  By their exponents.
+__device__ __forceinline__ bool two_float_holds(const StepArgs &a, const RowInfo &row, int r)
+{
+    const auto expo = [](double x) {
+        return (int)((__double_as_longlong(x) >> 52) & 0x7FF) - 1023;
+    };
+    const int ev = expo(a.v0[r]), ed = expo(a.dt), ec = expo(row.cells_per_length);
+    const auto inside = [](int e) { return e == -1023 || (e >= -60 && e <= 60); };
+    return inside(ev) && inside(ed) && inside(ec) && ev + ed + ec < 18;
+}
+
 // One segment of k_adj_seg: output cells [out0, out0 + stride) of a row.
 template <typename T, int ORDER>
 __device__ __forceinline__ void adj_segment(const StepArgs &a, const RowInfo &row,
@@ -276,10 +289,14 @@ __global__ void __launch_bounds__(kSegWarps * 32, sizeof(T) == 4 ? 6 : 4)
     pdl_wait();
     pdl_trigger();
     RowParams<T> P;
-    if constexpr (sizeof(T) == 4)
-        shift_params_two_float(a, row, r, seg0 == 0 && lane == 0, P);
-    else
+    if constexpr (sizeof(T) == 4) {
+        if (two_float_holds(a, row, r))
+            shift_params_two_float(a, row, r, seg0 == 0 && lane == 0, P);
+        else
+            shift_params<float>(a, row, r, false, P);
+    } else {
         P = pars[r];
+    }
     const int N = row.n, nsub = P.nsub;
     const int H = seg_halo<T>(nsub);
     const int stride = 32 * V - 2 * H;

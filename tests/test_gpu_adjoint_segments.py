@@ -87,3 +87,28 @@ def test_steps_in_a_row_equal_single_calls(n, k):
     torch.testing.assert_close(g_dv, gd, **close)
     with pytest.raises(ram.RamError):
         ram.steps(plan, q, q, k, v0, 1.0, dv=dv)
+
+
+@pytest.mark.parametrize("dt", [0.5, 1e-25, 1e-38, 1e35])
+def test_shifts_beyond_two_float_range(dt):
+    """FP32 rows whose shift, or a factor of it, two-float arithmetic does not hold to a
+    fraction of a cell take the FP64 shift (the suite's FP32 bar; a fraction wrong by
+    2^-10 of a cell, or a shift dropped, is far above it)."""
+    n, order = 1024, 3
+    x = wl.uniform_nodes(n, 0.0, 1.0)
+    shifts = np.array([0.37, 2.0**20 - 0.4, 2.0**21 + 0.7, -3.3e7, 2.0**33 + 0.6, 2.0**41 + 0.3])
+    rows = len(shifts)
+    v0 = shifts / n / dt
+    plan = ram.Plan(np.arange(rows + 1) * n, x, order=order, limiter=False, shared_mesh=True)
+    rng = np.random.default_rng(5)
+    q, g = (torch.tensor(a, dtype=torch.float32, device=DEV)
+            for a in rng.standard_normal((2, rows * n)))
+    gin = torch.empty_like(g)
+    ram.step_adjoint(plan, q, g, gin, torch.tensor(v0, device=DEV), dt)
+    assert plan.check_errors() == 0
+    got, qr, gr = (t.double().cpu().numpy() for t in (gin, q, g))
+    for r in range(rows):
+        sl = slice(r * n, (r + 1) * n)
+        ref, _ = oracle.step_adjoint(x, qr[sl], gr[sl], oracle.shift_from_velocity(v0[r], dt),
+                                     order, None, dt, 1)
+        assert np.abs(got[sl] - ref).sum() <= TOL["float32"] * np.abs(ref).sum(), r
