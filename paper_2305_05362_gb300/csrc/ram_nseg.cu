@@ -36,9 +36,8 @@
 // every cell at least 2^20 (a mean cell about 2^24).  Source and output widths,
 // positions and offsets all come from the same rounded nodes, so that what the
 // rounding does is to move the mesh by 2^-24 of a mean cell: the masses stay
-// consistent, and the results are as far from the exact ones as those of the
-// 64-bit positions of k_gwarp (relative 2-norm 1.0e-7 on the 512-row batch, against
-// 1.1e-7).
+// consistent, and the results are no further from the exact ones than those of the
+// per-order kernels' 64-bit positions (figures below).
 //
 // Why this form: at 16 bytes a cell the step is bound by the instructions it
 // issues and by the shared-memory passes of its gathers, not by DRAM (61% of the
@@ -46,17 +45,23 @@
 // the 512-row batch).  Five cells per lane, an odd number, keep every strided access
 // of the shared arrays free of bank conflicts (16-byte ones too), pay for the search
 // once per five edges, and form the stencil's differences and reciprocals once per
-// neighbour instead of once per use.  One body serves the three orders: as three
-// copies it missed the instruction cache (68 against 52 us).
+// neighbour instead of once per use.  One body serves the three orders: three copies
+// missed the instruction cache (68.2 us with them, 51.8 without, about 1 of the
+// difference from the plan's segment lengths, which came with it).
+//
+// The last quotient (Eq. 26) takes a correction step: it costs 2% (50.2 us against 49.3)
+// and keeps the error below the per-order kernels' over batches of rows (8.8e-8 against
+// 1.1e-7, relative 2-norm; 9.3e-8 without) and level with theirs on meshes graded 16:1
+// (0.77 to 1.13 times, 0.96 in the mean over 20 split steps; 0.79 to 1.19 without).
 //
 // Measured against the per-order kernels (k_params with k_gwarp, or k_general with a
 // residual), us per step: 512 rows of 64 to 65536 cells (5.3 M cells), no limiter,
-// 111.4 / 49.6, with a van Leer residual 203.4 / 66.0; 1000 rows (9.5 M) limited
-// 196.0 / 87.8; one row of 4096 cells with a residual 14.3 / 7.7.  Tried (when the batch
-// took 52.0): seven cells
-// per lane 57.5 (512 rows), seven or five CTAs per SM instead of six 52.9 and 52.9, the
-// lane's edges by side-by-side halvings instead of the walk 54.7, a loop without the
-// two predicated steps 54.9, the next node's position kept across edges 55.6.
+// 112.6 / 50.2, with a van Leer residual 204.8 / 67.1; 1000 rows (9.5 M) limited
+// 198.6 / 90.3; one row of 4096 cells with a residual 14.3 / 7.8.  Tried (when the batch
+// took 52.0): seven cells per lane 57.5 (512 rows), seven or five CTAs per SM instead of
+// six 52.9 and 52.9, the lane's edges by side-by-side halvings instead of the walk 54.7,
+// a loop without the two predicated steps 54.9, the next node's position kept across
+// edges 55.6; when it took 49.4, the walk by pointers 51.6.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -431,10 +436,14 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
         for (int i = 0; i < kV; ++i) {
             const int j = b + i;
             // Eq. 18: the start of the right source cell less that of the left one, plus
-            // the cells passed from the left one on; Eq. 26
-            if (j >= from && j < last)
-                sP[j] = (mass[i] + (G[i + 1] - G[i])) *
-                        rcp_approx((float)(xo[i + 1] - xo[i]) * g.scale);
+            // the cells passed from the left one on; Eq. 26, the quotient by the
+            // approximate reciprocal and one correction
+            if (j >= from && j < last) {
+                const float m = mass[i] + (G[i + 1] - G[i]);
+                const float h = (float)(xo[i + 1] - xo[i]) * g.scale, rh = rcp_approx(h);
+                const float v = m * rh;
+                sP[j] = fmaf(fmaf(-v, h, m), rh, v);
+            }
         }
         if (least == 0) {
             // an edge on a node: a cell whose edges both are, on those of one source cell,
