@@ -168,7 +168,8 @@ def _traffic(kernel_key):
 
 
 def _kernel_name(tuning):
-    """The FP32 uniform-row kernel (order 3) the tuning selects, as ncu names it."""
+    """The FP32 uniform-row kernel (order 3) the tuning selects, as ncu names it (the ring
+    kernel without its last argument, the A4 form)."""
     k = tuning["uniform_kernel_f32"]
     if k == 0:
         return "k_rows<float,3,%d>" % tuning["rows_cells_per_thread_f32"]

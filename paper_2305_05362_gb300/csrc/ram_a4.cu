@@ -11,7 +11,9 @@
 // rows of 25 cells or more the sum is taken over |m| <= 12 on the infinite-lattice
 // weights A r^|m| (the images are below FP64 rounding); shorter rows take the
 // exact periodic weights.  Both kernels run one thread per cell over the plan's
-// tiles of the order-3 uniform rows.
+// tiles of the order-3 uniform rows.  Steps whose rows all take a warp-segment kernel
+// do the same in its registers (ram_useg.cu); these kernels, with the step's own
+// between them, take the others (short or misaligned rows, other kernels by tuning).
 #include <cuda_runtime.h>
 
 #include "ram_device.cuh"

@@ -24,7 +24,7 @@
 //
 // Bound by the FP64 pipe in double precision: carrying the limited reconstruction's
 // value with its derivatives along five stencil cells, every weight with range-checked
-// divides, took 685 us on 64 rows (597 K cells, PPM), the passes below 146.
+// divides, took 685 us on 64 rows (597 K cells, PPM, limited), the passes below 184.
 //
 // The donor residual sub-steps (Eq. 6) with per-cell widths have the transpose
 //   lf_j = g_j / dx_j - g_{j-1} / dx_{j-1},  g_up(j) += c_j lf_j,

@@ -1,9 +1,12 @@
 // RAM step on rows with their own non-uniform mesh (Sec. 3 on an arbitrary
 // periodic mesh), and the per-row mass diagnostic.
 //
-// Steps without a residual run k_gwarp (below): warps split each tile, each lane
-// locates its own edges and gathers the source stencils from the cache, with no
-// shared memory or barriers.  Steps with a residual run k_general:
+// These kernels take the rows that the warp-segment kernels (ram_nseg.cu,
+// ram_nseg_f64.cu) do not: shorter than kNsegMinCells, or graded beyond one of their
+// windows, and FP32 rows where the plan's tuning asks for them.  Steps without a
+// residual run k_gwarp (below): warps split each tile, each lane locates its own edges
+// and gathers the source stencils from the cache, with no shared memory or barriers.
+// Steps with a residual run k_general:
 //
 // One CTA per tile of output cells.  The tile's source window -- the source
 // cells its shifted edges land in, plus the reconstruction halo -- is found

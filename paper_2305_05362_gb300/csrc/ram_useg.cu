@@ -466,11 +466,11 @@ struct RingLayout {
 // a lane for dv, 4 for the window, whose start the shift leaves on any word -- so that
 // every lane's cells lie at the same 16-byte boundary of the stage (with 16-byte copies
 // each lane read five vectors and moved its cells into place by the offset in them:
-// 15.2 us on the 1024 x 4096 disk and 312.9 on the 8192 x 16384 one, 14.8 and 305.2 so).  A warp reads a stage into registers, refills it at once with the
-// copies of its next segment and computes.  The warps of a row take its segments
-// from a counter in shared memory as they issue the copies, so a warp on a
-// crowded scheduler takes fewer of them and the row's CTA finishes with its
-// warps.  The row's shift parameters are formed in the kernel
+// 15.2 us on the 1024 x 4096 disk and 312.9 on the 8192 x 16384 one, 14.8 and 305.2 so).
+// A warp reads a stage into registers, refills it at once with the copies of its next
+// segment and computes.  The warps of a row take its segments from a counter in
+// shared memory as they issue the copies, so a warp on a crowded scheduler takes
+// fewer of them and the row's CTA finishes with its warps.  The row's shift parameters are formed in the kernel
 // (shift_params_two_float), so no parameter kernel runs before it when every row
 // of the step takes this kernel; the phase is then advanced here too
 // (a.row_phase).  FP32 rows of at least 32 V + 12 cells.
@@ -479,7 +479,7 @@ struct RingLayout {
 // registers before the remap and the point values recovered after it (a4_average,
 // a4_points), with a wider halo: one launch and 12 bytes a cell, against four kernels
 // that passed the field through memory between them (512 x 4096 cells with a
-// residual, steps back to back: 45.4 and 9.9 us).
+// residual, steps back to back: 46.9 and 10.3 us).
 template <int ORDER, int V, bool LIM, bool VL, bool A4>
 __global__ void __launch_bounds__(256, 3)
     k_useg_ring(StepArgs a, const int32_t *row_ids)
