@@ -24,10 +24,10 @@
  *  - Device pointers are device memory of the plan's device.  The caller owns
  *    every cell, velocity, shift, phase and gradient buffer; the plan owns its
  *    copy of the mesh, its tile lists and its device error word.
- *  - The step entry points (ram_shift, ram_residual_upwind, ram_step,
- *    ram_step_adjoint, ram_row_mass) only enqueue kernels on `stream`: they
- *    never allocate and never synchronise, so they may be captured in a CUDA
- *    graph.  They validate host-visible arguments synchronously and return an
+ *  - The step entry points (ram_shift, ram_residual_upwind, ram_step, ram_steps,
+ *    ram_step_adjoint, ram_steps_adjoint, ram_radial_upwind, ram_row_mass) only
+ *    enqueue kernels on `stream`: they never allocate and never synchronise, so
+ *    they may be captured in a CUDA graph.  They validate host-visible arguments synchronously and return an
  *    error without launching anything.  Conditions found on the device (CFL
  *    above 1 in the residual step, a non-finite shift, an out-of-range sub-step
  *    count, a wait that timed out) set bits in the plan's error word, which
@@ -98,7 +98,8 @@ typedef struct {
  * Sec. 3.2 index search).  Validates the mesh, copies it to the device in the
  * plan's own layout, classifies rows (uniform rows take the O(1) index of
  * Sec. 3.2.1), builds the tile lists and allocates the error word.  Host
- * synchronous; the only entry point besides ram_plan_autotune that allocates.
+ * synchronous; besides it only ram_plan_set_density, ram_plan_set_tiling,
+ * ram_plan_set_tuning and ram_plan_autotune allocate.
  * On failure *out is NULL and nothing is leaked. */
 ram_status ram_plan_mesh(const ram_mesh_desc *desc, int device, ram_plan *out);
 
@@ -163,7 +164,8 @@ ram_status ram_step(ram_plan plan, ram_dtype dtype, const void *q_in, void *q_ou
  * as the forward ram_step) and the cotangent g_out of the step output, writes
  * g_in = J^T g_out and, when g_dv is not NULL, ADDS d<g_out, out>/d dv into g_dv
  * (device, same packing and dtype as dv).  At dv_j == 0 the upwind side of the
- * flux derivative is the left cell.  dv_iface NULL -> no residual step. */
+ * flux derivative is the left cell.  dv_iface NULL -> no residual step.  The shift of
+ * FP32 uniform rows is formed as in ram_step, beyond 2^20 cells in FP64. */
 ram_status ram_step_adjoint(ram_plan plan, ram_dtype dtype, const void *q_in,
                             const void *g_out, void *g_in, const double *v0, double dt,
                             const void *dv_iface, void *g_dv, const int32_t *nsub,
@@ -269,8 +271,8 @@ typedef struct {
                                            lane and segment (8 needs rows >= 520 cells) */
     int32_t seg_variant_f32;            /* warp-segment kernel, FP32: 0 = one segment in
                                            flight per warp, 1 = the loads of a warp's next
-                                           segment in flight while it computes, 2 = a ring
-                                           of 2 shared-memory stages per warp, the row's
+                                           segment in flight while it computes, 2 = a
+                                           shared-memory stage per warp, the row's
                                            segments handed out by a counter as the warps
                                            issue their copies, its shift parameters
                                            formed in the kernel (no parameter kernel
