@@ -207,6 +207,8 @@ def _step_pointers(plan: "Plan", cells, rows, dv=None, nsub=None):
     of them is not what the plan takes (the caller then finds out which)."""
     import torch
     n, nr, dev = plan.n_cells, plan.n_rows, plan.device
+    if cells[0][1] is None:
+        return None
     dtype = cells[0][1].dtype
     if dtype is not torch.float32 and dtype is not torch.float64:
         return None

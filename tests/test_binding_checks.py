@@ -81,6 +81,21 @@ def test_shift_residual_adjoint_mass_refusals(plan):
         ram.row_mass(plan, _f32(40), _f64(3))
 
 
+def test_missing_tensors_are_named(plan):
+    """A missing tensor is refused by name, the first one too (whose dtype the others are
+    checked against)."""
+    q, v0 = _f32(40), _f64(4)
+    with pytest.raises(ValueError, match="q_in is required"):
+        ram.step(plan, None, q, v0, 0.1)
+    with pytest.raises(ValueError, match="q_in is required"):
+        ram.shift(plan, None, q, v0)
+    with pytest.raises(ValueError, match="is required"):
+        ram.step_adjoint(plan, q, None, q, v0, 0.1)
+    for args in ((q, None, v0), (q, q, None)):
+        with pytest.raises(ValueError, match="is required"):
+            ram.step(plan, *args, 0.1)
+
+
 def test_noalloc_refusals():
     q, out = _f32(8 * 512), _f32(8 * 512)
     v0 = _f64(8)
