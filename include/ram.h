@@ -295,13 +295,14 @@ ram_status ram_plan_set_tuning(ram_plan plan, const ram_tuning *tuning);
  * on the caller's buffers -- the arguments of ram_step, without the phase --
  * with CUDA events on `stream` (`reps` timed steps per candidate) and keeps the
  * fastest in the plan.  Candidates: for uniform rows the warp-segment kernel
- * (3, 4, 6 or 8 warps per row CTA; FP32: with and without prefetch),
+ * (FP32: its three variants with 3, 4, 6 or 8 warps per row CTA),
  * for FP32 the streaming-warp kernel with 4 or 8 cells per lane, and the
  * persistent whole-row kernel with (cells per thread, CTAs per SM) in
  * {5,7,9,11,15} x {2,3,4} as the register budget allows; tile cells
- * {256,512,1024,2048} x threads {128,256,512} of the tiled kernels; for FP32
- * rows with their own mesh, the warp-segment kernel against the per-order
- * kernels.  Host synchronous; overwrites q_out. */
+ * {256,512,1024,2048} x threads {128,256,512} when the plan has rows that take
+ * the tiled kernels; for FP32 rows with their own mesh, the warp-segment kernel
+ * against the per-order kernels.  An FP64 run leaves the _f32 fields and seg_warps
+ * as they are.  Host synchronous; overwrites q_out. */
 ram_status ram_plan_autotune(ram_plan plan, ram_dtype dtype, const void *q_in, void *q_out,
                              const double *v0, double dt, const void *dv_iface,
                              ram_scheme scheme, const int32_t *nsub, int32_t reps,

@@ -115,23 +115,27 @@ extern "C" ram_status ram_plan_autotune(ram_plan plan, ram_dtype dtype, const vo
         return r;
     };
     const int d = dtype == RAM_F64 ? 1 : 0;
-    bool any_rows = false, any_tiles = false;
+    bool any_rows = false, any_seg = false;
     for (int o = 2; o <= 4; ++o) {
         any_rows |= !p->rows_fit_h[d][o].empty();
-        any_tiles |= !p->tiles_rest_h[d][o].empty() || !p->tiles_general_h[o].empty();
+        any_seg |= !p->rows_seg_h[d][o].empty();
     }
-    bool any_seg = false;
-    for (int o = 2; o <= 4; ++o) any_seg |= !p->rows_seg_h[d][o].empty();
     if (any_rows || any_seg) {
         // candidates: (kernel, cells per thread)
         int best_k = p->uniform_kernel[d], best_v = p->rows_v[d], best_c = p->rows_cps[d];
         int best_sv = p->stream_v, best_gv = p->seg_variant, best_gw = p->seg_warps;
         float best = 3.4e38f;
-        if (any_seg)
-            for (int gv = 0; gv <= (d == 0 ? 2 : 0) && st == RAM_OK; ++gv)
+        if (any_seg && d == 1) {
+            // one form and one shape (seg_variant and seg_warps are the FP32 kernel's)
+            p->uniform_kernel[1] = 1;
+            st = time_once(&best);
+            if (st == RAM_OK) best_k = 1;
+        }
+        if (any_seg && d == 0)
+            for (int gv = 0; gv <= 2 && st == RAM_OK; ++gv)
                 for (int gw : {3, 4, 6, 8}) {
                     if (st != RAM_OK) break;
-                    p->uniform_kernel[d] = 1;
+                    p->uniform_kernel[0] = 1;
                     p->seg_variant = gv;
                     p->seg_warps = gw;
                     float ms = 0;
@@ -179,6 +183,14 @@ extern "C" ram_status ram_plan_autotune(ram_plan plan, ram_dtype dtype, const vo
         p->stream_v = best_sv;
         p->seg_variant = best_gv;
         p->seg_warps = best_gw;
+    }
+    // rows of the tiled kernels (rows of the other kernels do not see the tile shape)
+    bool any_tiles = false;
+    for (int o = 2; o <= 4; ++o) {
+        any_tiles |= p->uniform_kernel[d] == 0 ? !p->tiles_rest_h[d][o].empty()
+                                               : !p->tiles_rest_seg_h[d][o].empty();
+        any_tiles |= d == 1 || p->nu_kernel == 1 ? !p->tiles_general32_h[o].empty()
+                                                 : !p->tiles_general_h[o].empty();
     }
     if (any_tiles && st == RAM_OK) {
         const int tcs[] = {256, 512, 1024, 2048};
