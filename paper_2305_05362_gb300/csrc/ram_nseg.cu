@@ -37,7 +37,10 @@
 // positions and offsets all come from the same rounded nodes, so that what the
 // rounding does is to move the mesh by 2^-24 of a mean cell: the masses stay
 // consistent, and the results are no further from the exact ones than those of the
-// per-order kernels' 64-bit positions (figures below).
+// per-order kernels' 64-bit positions (figures below).  The shift is not rounded: it is
+// the same at every step of a steady rotation, so that its rounding would add up.  It is
+// a whole number of units, rounded up, and a rest below a unit that every offset in a
+// cell takes along.
 //
 // Why this form: at 16 bytes a cell the step is bound by the instructions it
 // issues and by the shared-memory passes of its gathers, not by DRAM (61% of the
@@ -213,7 +216,8 @@ struct Item {
     int32_t nsub;
     float cf;                  // sub-step length
     float scale;               // position units -> the widths' units, about mean widths
-    uint32_t S32, period;      // shift and period in position units (mod 2^32)
+    float rem;                 // what S32 is more than the shift, in the widths' units
+    uint32_t S32, period;      // shift (rounded up) and period in position units (mod 2^32)
 };
 
 struct SegCtx {
@@ -223,8 +227,8 @@ struct SegCtx {
     const float *dvp, *dx;
     int N, H, nsub, lane, hi;  // hi: first window node past the cells an edge may lie in
     bool vl;
-    float scale, cf;
-    uint32_t S32, period;      // shift and period in position units (mod 2^32)
+    float scale, rem, cf;      // as in Item
+    uint32_t S32, period;
     int *err;
 };
 
@@ -319,7 +323,8 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
     }
     cp_async_commit();
 
-    uint32_t off = 0;       // position of a shifted node in the window: x - off
+    uint32_t off = 0;       // position of a shifted node in the window: x - off (and g.rem)
+    bool before = false;    // edge 0 is before the window's first source cell
     int from = 0;           // first edge that is left
     bool first = true;
     while (true) {
@@ -351,10 +356,11 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
         }
         __syncwarp();
         if (first) {
-            // the first edge lies in source cell p, up to the rounding of the shift
+            // the first edge lies in source cell p, or, as the nodes are rounded, up to a
+            // unit before it: then it is at the cell's node
             off = (x_first - g.S32 - xb) & (g.period - 1u);
-            if (off >= kPast - 1u || off == g.period - 1u) off = 0;
-            off = x_first - off;
+            before = off == g.period - 1u;
+            off = before ? x_first + 1u : x_first - off;
             // the window's values and nodes are in use no more
             advance();
             copies();
@@ -370,6 +376,7 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
         int w = kHR;
         uint32_t rw = 0;  // position of node w
         uint32_t ry = min(xo[0] - off, kPast - 1u);
+        if (before && b == 0) ry = 0;
         // the last node at or left of the edge: the nodes past the window are kPast,
         // so no bound is needed
 #pragma unroll
@@ -385,7 +392,7 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
             const uint32_t d = ry - rw;
             we[i] = w;
             de[i] = d;
-            const float x = (float)d * g.scale;
+            const float x = fmaf((float)d, g.scale, g.rem);
             float4 c = sC[w];
             if (order == 4) {
                 c.z = fmaf(x, c.w, c.z);
@@ -445,7 +452,7 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
                 sP[j] = fmaf(fmaf(-v, h, m), rh, v);
             }
         }
-        if (least == 0) {
+        if (least == 0 && g.rem == 0.f) {
             // an edge on a node: a cell whose edges both are, on those of one source cell,
             // takes its value unchanged
 #pragma unroll
@@ -608,13 +615,16 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
         it.p = locate_cell(X, row.n, a.buckets + row.bucket_off, row.bucket_bits, a.density,
                            row.density, xe - S);
         it.S = S;
-        it.S32 = (uint32_t)((S + (qs > 0 ? 1ull << (qs - 1) : 0ull)) >> qs);
+        // the shift in whole units, rounded up, and the rest
+        const uint64_t low = S & ((1ull << qs) - 1ull);
+        it.S32 = (uint32_t)(S >> qs) + (low != 0 ? 1u : 0u);
         if (qs > 32) it.S32 &= (1u << (64 - qs)) - 1u;
         it.period = qs > 32 ? 1u << (64 - qs) : 0u;
         it.nsub = P.nsub;
         it.cf = P.cf;
         // a power of two, so that widths and offsets round once; a mean cell is in [1, 2)
         it.scale = __int_as_float((127 + qs - 64 + 32 - __clz(row.n)) << 23);
+        it.rem = low != 0 ? it.scale * (1.f - ldexpf((float)low, -qs)) : 0.f;
         s_item[tid] = it;
     }
     __syncthreads();
@@ -684,6 +694,7 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
         g.hi = kHR + min(kWin - 2 * kHR, 2 * g.N - 1);
         g.vl = R == 2;
         g.scale = it.scale;
+        g.rem = it.rem;
         g.cf = it.cf;
         g.S32 = it.S32;
         g.period = it.period;

@@ -1,0 +1,59 @@
+"""FP32 rows with their own mesh on the warp-segment kernel, where its 32-bit positions,
+its plain sums and its limiters could differ from the per-order kernels that hold 64-bit
+positions and compensated sums: shifts of about one position unit, output cells over many
+source cells, values that are not finite, and magnitudes far from 1."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+from paper_2305_05362_gb300 import ram, workloads as wl
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _bump(n):
+    return wl.bump_nodes(n, -np.pi, np.pi, 0.1387, 0.2773, 15.0)
+
+
+def _plan(x, kernel=1, **kw):
+    plan = ram.Plan([0, x.size - 1], x, **kw)
+    assert plan.info().n_nseg_rows == 1
+    t = plan.tuning()
+    t.nonuniform_kernel_f32 = kernel
+    plan.set_tuning(t)
+    return plan
+
+
+def _step(plan, q, s, dt=0.1, dv=None, scheme=ram.VANLEER, nsub=1, n_steps=1):
+    a = torch.tensor(np.asarray(q), dtype=torch.float32, device=DEV)
+    b = torch.empty_like(a)
+    v0 = torch.tensor([s / dt], dtype=torch.float64, device=DEV)
+    d = None if dv is None else torch.tensor(np.asarray(dv), dtype=torch.float32, device=DEV)
+    ns = None if dv is None else torch.tensor([nsub], dtype=torch.int32, device=DEV)
+    for _ in range(n_steps):
+        ram.step(plan, a, b, v0, dt, dv=d, scheme=scheme, nsub=ns)
+        a, b = b, a
+    return a.double().cpu().numpy()
+
+
+@pytest.mark.parametrize("units", [0.3, 0.8, 1.45, 2.55, 7.3])
+@pytest.mark.parametrize("n", [510, 1533])
+@pytest.mark.parametrize("order", [2, 3])
+def test_shifts_of_about_one_position_unit(order, n, units):
+    """A position unit is up to 2^-20 of the narrowest cell.  A top-hat of height 1 moved
+    left by about that much puts s / dx into the empty cell beside its left end: one
+    product and one quotient in FP32, within 1e-5 relative, and 1e-4 for what the oracle's
+    FP64 positions leave of a shift of 1e-9 cells."""
+    x = _bump(n)
+    dx = np.diff(x)
+    xc = 0.5 * (x[1:] + x[:-1])
+    q = (np.abs(xc) < 0.08).astype(np.float64)  # its ends lie in the narrow cells
+    beside = np.flatnonzero(q)[0] - 1
+    s = -units * dx.min() * 2.0 ** -20
+    got = _step(_plan(x, order=order), q, s)[beside]
+    ref = oracle.step(x, q, oracle.shift_from_velocity(s / 0.1, 0.1), order, True)[beside]
+    assert ref > 0.0
+    assert abs(got - ref) <= 1e-4 * ref
