@@ -417,10 +417,15 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
                 ++w;
                 rw = r;
             }
+            // more where the mesh under the segment is finer: compensated (Kahan), as their
+            // number is only bounded by the window's
+            float lost = 0.f;
             while (true) {
                 r = sR[w + 1];
                 if (r > ry) break;
-                m += sM[w];
+                const float v = sM[w] - lost, t = m + v;
+                lost = (t - m) - v;
+                m = t;
                 ++w;
                 rw = r;
             }

@@ -57,3 +57,26 @@ def test_shifts_of_about_one_position_unit(order, n, units):
     ref = oracle.step(x, q, oracle.shift_from_velocity(s / 0.1, 0.1), order, True)[beside]
     assert ref > 0.0
     assert abs(got - ref) <= 1e-4 * ref
+
+
+@pytest.mark.parametrize("with_dv", [False, True])
+def test_output_cells_over_many_source_cells(with_dv):
+    """Wide cells over up to 144 narrow ones: their masses are sums of that many cells.
+    Against the FP64 oracle on the same values, the wide cells within 2^-22 (products,
+    their sum kept in two floats, one quotient: a few half units of 2^-24)."""
+    rng = np.random.default_rng(8)
+    w = np.ones(2000)
+    w[1000:1010] = 140.0
+    x = np.concatenate([[0.0], np.cumsum(w)]) / w.sum()
+    n = w.size
+    q = (1.0 + rng.random(n)).astype(np.float32).astype(np.float64)
+    wide = np.flatnonzero(w > 1.0)
+    dv = np.zeros(n) if with_dv else None
+    for order in (2, 3):
+        plan = _plan(x, order=order)
+        for k in range(8):
+            s = (1400.0 + 37.3 * k) / w.sum()  # under the wide cells: narrow ones
+            got = _step(plan, q, s, dv=dv)
+            ref = oracle.step(x, q, oracle.shift_from_velocity(s / 0.1, 0.1), order, True)
+            err = np.abs(got - ref)[wide] / ref[wide]
+            assert err.max() <= 2.0 ** -22, (order, k, err.max() * 2.0 ** 24)
