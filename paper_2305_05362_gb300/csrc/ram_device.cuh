@@ -39,6 +39,19 @@ __device__ __forceinline__ float minxs(float a, float b)
     asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
     return d;
 }
+// the same, NaN where one of them is
+__device__ __forceinline__ float minxs_nan(float a, float b)
+{
+    float d;
+    asm("min.NaN.xorsign.abs.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float d;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+    return d;
+}
 // max(|a|, |b|, |c|)
 __device__ __forceinline__ float max_abs3(float a, float b, float c)
 {

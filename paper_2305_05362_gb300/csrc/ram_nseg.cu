@@ -143,7 +143,8 @@ __device__ __forceinline__ void reconstruct(const float (&q)[kV + 4], const floa
         for (int t = 1; t < kV + 3; ++t) {
             const float num = fmaf(s2[t - 1] + h[t - 1], D2[t], (s2[t] + h[t + 1]) * D2[t - 1]);
             dq[t] = h[t] * num * rcp_approx(s2[t - 1] + h[t + 1]);
-            if (LIM) dq[t] = minxs(dq[t], fmaxf(2.f * minxs(up[t - 1], up[t]), 0.f));
+            // (beside a NaN: 0)
+            if (LIM) dq[t] = minxs(dq[t], fmaxf(2.f * minxs_nan(up[t - 1], up[t]), 0.f));
         }
         // <Q>_{k+1/2} - Q_k of App. A.1 (weights read with sums of widths), one
         // reciprocal of the common denominator (2 h0 + h1)(h0 + 2 h1)(h- + h0 + h1 + h2)
@@ -157,14 +158,15 @@ __device__ __forceinline__ void reconstruct(const float (&q)[kV + 4], const floa
             fa[t] = fmaf(h[t], D2[t], n * rcp_approx(B * C * S4));
         }
         // with a = QR - Q, b = Q - QL: G = (Q - b) d + (2b - a) d^2 / h + (a - b) d^3 / h^2;
-        // limited (App. A.2, second stage): a' = median(0, a, 2b), b' = median(0, b, 2a)
+        // limited (App. A.2, second stage): a' = median(0, a, 2b), b' = median(0, b, 2a); a
+        // NaN on one side makes the cell's profile NaN, as it does unlimited
 #pragma unroll
         for (int i = 0; i < kV; ++i) {
             const int t = i + 2;
             float a = fa[t], b = up[t - 1] - fa[t - 1];
             if (LIM) {
-                const float a1 = xorsign(fmaxf(minxs(a, b + b), 0.f), a);
-                b = xorsign(fmaxf(minxs(b, a + a), 0.f), b);
+                const float a1 = xorsign(max_nan(minxs_nan(a, b + b), 0.f), a);
+                b = xorsign(max_nan(minxs_nan(b, a + a), 0.f), b);
                 a = a1;
             }
             const float ih = rcp_approx(h[t]);

@@ -80,3 +80,29 @@ def test_output_cells_over_many_source_cells(with_dv):
             ref = oracle.step(x, q, oracle.shift_from_velocity(s / 0.1, 0.1), order, True)
             err = np.abs(got - ref)[wide] / ref[wide]
             assert err.max() <= 2.0 ** -22, (order, k, err.max() * 2.0 ** 24)
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("order,limiter", [(2, True), (2, False), (3, True), (3, False),
+                                           (4, True), (4, False)])
+def test_values_that_are_not_finite(value, order, limiter):
+    """A NaN reaches the cells that it reaches with the per-order kernel, an infinity none
+    that neither of them reaches there; where both kernels' results are finite they
+    agree."""
+    n = 1533
+    x = wl.random_nodes(n, seed=n + 5)
+    q = 1.0 + np.random.default_rng(4).random(n)
+
+    def run(kernel, v):
+        plan = _plan(x, kernel, order=order, limiter=limiter)
+        out = _step(plan, np.where(np.arange(n) == 700, v, q), 0.2)
+        assert plan.check_errors() == 0
+        return out
+
+    got, ref, nan = run(1, value), run(0, value), run(0, np.nan)
+    if np.isnan(value):
+        np.testing.assert_array_equal(np.isfinite(got), np.isfinite(ref))
+    assert not np.isfinite(got).all()
+    assert np.isfinite(got[np.isfinite(nan) & np.isfinite(ref)]).all()
+    fine = np.isfinite(got) & np.isfinite(ref)
+    np.testing.assert_allclose(got[fine], ref[fine], rtol=1e-5)
