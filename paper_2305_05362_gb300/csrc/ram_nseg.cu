@@ -99,6 +99,17 @@ constexpr int kOffH = kOffV + kWin + 4;      // widths of the segment's cells (r
 constexpr int kWordsResid = kOffH + kWin + 4;
 static_assert(kOffC % 4 == 0 && kWords % 4 == 0 && kWordsResid % 4 == 0, "16-byte aligned");
 
+// x y / (x + y) where x and y have one sign, else 0, as (x + y) times the shares x / (x + y)
+// and y / (x + y), each cut to [0, 1]: of opposite signs one share is negative.  (The
+// product x y would leave the range of FP32 below 1e-22 and above 1e19.)  Beside a NaN or
+// an infinity it is 0: the cut takes a NaN to 0.
+__device__ __forceinline__ float harmonic(float x, float y)
+{
+    const float s = x + y, r = rcp_approx(s);
+    const float p = __saturatef(x * r) * __saturatef(y * r);
+    return p > 0.f ? p * s : 0.f;
+}
+
 // Coefficients of the in-cell cumulative G(d) = d (c0 + d (c1 + d (c2 + d c3))) of
 // the lane's cells, d the distance from the cell's left node in the units of h
 // (mean widths).  q[t], h[t]: cells -2 .. kV + 1 of the lane at t = 0 .. kV + 3; the
@@ -113,18 +124,19 @@ __device__ __forceinline__ void reconstruct(const float (&q)[kV + 4], const floa
         s2[t] = h[t] + h[t + 1];
         up[t] = q[t + 1] - q[t];
     }
+    float D2[kV + 3];  // (Q_{t+1} - Q_t) / (h_t + h_{t+1})
+#pragma unroll
+    for (int t = 0; t < kV + 3; ++t) D2[t] = up[t] * rcp_approx(s2[t]);
     if (ORDER == 2) {
         // G = q d + sigma (d^2 - h d) / 2.  Limited: the van Leer harmonic mean of the
-        // one-sided slopes over centre spacings, zero at an extremum (sigma / 2 =
-        // 2 dl dr / (dl (h0 + h+) + dr (h- + h0))); else the centred slope
+        // one-sided slopes over centre spacings, 2 D2 each, zero at an extremum; else the
+        // centred slope
 #pragma unroll
         for (int i = 0; i < kV; ++i) {
             const int t = i + 2;
             float half;
             if (LIM) {
-                const float p = up[t - 1] * up[t];
-                const float den = up[t - 1] * s2[t] + up[t] * s2[t - 1];
-                half = p > 0.f ? 2.f * p * rcp_approx(den) : 0.f;
+                half = 2.f * harmonic(D2[t - 1], D2[t]);
             } else {
                 half = (up[t - 1] + up[t]) * rcp_approx(s2[t - 1] + s2[t]);
             }
@@ -132,9 +144,6 @@ __device__ __forceinline__ void reconstruct(const float (&q)[kV + 4], const floa
         }
         return;
     }
-    float D2[kV + 3];  // (Q_{t+1} - Q_t) / (h_t + h_{t+1})
-#pragma unroll
-    for (int t = 0; t < kV + 3; ++t) D2[t] = up[t] * rcp_approx(s2[t]);
     if (ORDER == 3) {
         // delta<Q> of App. A.1, b / (a + b + c) [(2a + b) D2_k + (b + 2c) D2_{k-1}], limited
         // by the first stage of App. A.2
@@ -217,7 +226,8 @@ struct Item {
     int32_t order;
     int32_t p;                 // source cell of the first edge (halo included)
     int32_t nsub;
-    float cf;                  // sub-step length
+    float wscale;              // 2^k: a mean width times it is in (1, 2]
+    float cf;                  // sub-step length, times wscale
     float scale;               // position units -> the widths' units, about mean widths
     float rem;                 // what S32 is more than the shift, in the widths' units
     uint32_t S32, period;      // shift (rounded up) and period in position units (mod 2^32)
@@ -516,48 +526,50 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
         cp_async_wait<1>();  // dv (the group before the next segment's)
         __syncwarp();
         const unsigned full = 0xffffffffu;
-        const float cf = it.cf;
+        const float cf = it.cf, wscale = it.wscale;
         float cur[kV], c[kV], h[kV], rh[kV];
 #pragma unroll
         for (int i = 0; i < kV; ++i) {
             cur[i] = sP[b + i];
-            c[i] = sV[b + i] * cf;  // signed length swept by node i in a sub-step
-            h[i] = sV[kOffH - kOffV + b + i];
+            c[i] = sV[b + i] * cf;  // signed length swept by node i in a sub-step, scaled
+            h[i] = sV[kOffH - kOffV + b + i] * wscale;
             rh[i] = rcp_approx(h[i]);
         }
-        const float hm = __shfl_up_sync(full, h[kV - 1], 1), hp = __shfl_down_sync(full, h[0], 1);
+        const float hm = __shfl_up_sync(full, h[kV - 1], 1);
         const int R = g.vl ? 2 : 1;
         bool bad = false;
+        float rs[kV + 1], wc[kV];  // 1 / (both widths at face i), twice the midpoint's offset
 #pragma unroll
-        for (int i = 0; i < kV; ++i)
-            bad |= b + i >= R && b + i <= ne - R &&
-                   fabsf(c[i]) > (c[i] > 0.f ? (i ? h[i - 1] : hm) : h[i]);
+        for (int i = 0; i < kV; ++i) {
+            const float hl = i ? h[i - 1] : hm;
+            const bool pos = c[i] > 0.f;
+            bad |= b + i >= R && b + i <= ne - R && fabsf(c[i]) > (pos ? hl : h[i]);
+            rs[i] = rcp_approx(hl + h[i]);
+            wc[i] = 2.f * ((pos ? hl : -h[i]) - c[i]);
+        }
+        rs[kV] = __shfl_down_sync(full, rs[0], 1);
         if (__any_sync(full, bad) && lane == 0) atomicOr(g.err, ERR_CFL);
         for (int ks = 0, nsub = it.nsub; ks < nsub; ++ks) {
             const float zl = __shfl_up_sync(full, cur[kV - 1], 1);
             float F[kV];
             if (g.vl) {
-                // half slopes per unit length (van Leer harmonic mean, centre spacings)
+                // a quarter of the slopes (van Leer harmonic mean, centre spacings)
                 const float zr = __shfl_down_sync(full, cur[0], 1);
-                float s[kV];
+                float s[kV], Dl = (cur[0] - zl) * rs[0];
 #pragma unroll
                 for (int i = 0; i < kV; ++i) {
-                    const float dl = cur[i] - (i ? cur[i - 1] : zl);
-                    const float dr = (i < kV - 1 ? cur[i + 1] : zr) - cur[i];
-                    const float sl = (i ? h[i - 1] : hm) + h[i];
-                    const float sr = h[i] + (i < kV - 1 ? h[i + 1] : hp);
-                    const float pr = dl * dr;
-                    s[i] = pr > 0.f ? 2.f * pr * rcp_approx(fmaf(dl, sr, dr * sl)) : 0.f;
+                    const float Dr = ((i < kV - 1 ? cur[i + 1] : zr) - cur[i]) * rs[i + 1];
+                    s[i] = harmonic(Dl, Dr);
+                    Dl = Dr;
                 }
-                const float slp = __shfl_up_sync(full, s[kV - 1], 1);
+                const float sl = __shfl_up_sync(full, s[kV - 1], 1);
 #pragma unroll
                 for (int i = 0; i < kV; ++i) {
                     // the upwind cell's value at the middle of the swept length
                     const bool pos = c[i] > 0.f;
                     const float zu = pos ? (i ? cur[i - 1] : zl) : cur[i];
-                    const float su = pos ? (i ? s[i - 1] : slp) : -s[i];
-                    const float hu = pos ? (i ? h[i - 1] : hm) : h[i];
-                    F[i] = c[i] * fmaf(su, hu - fabsf(c[i]), zu);
+                    const float su = pos ? (i ? s[i - 1] : sl) : s[i];
+                    F[i] = c[i] * fmaf(su, wc[i], zu);
                 }
             } else {
 #pragma unroll
@@ -632,7 +644,9 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
         if (qs > 32) it.S32 &= (1u << (64 - qs)) - 1u;
         it.period = qs > 32 ? 1u << (64 - qs) : 0u;
         it.nsub = P.nsub;
-        it.cf = P.cf;
+        const int ex = ((__double2hiint(row.cells_per_length) >> 20) & 0x7ff) - 1023;
+        it.wscale = __int_as_float((127 + min(max(ex + 1, -126), 127)) << 23);
+        it.cf = P.cf * it.wscale;
         // a power of two, so that widths and offsets round once; a mean cell is in [1, 2)
         it.scale = __int_as_float((127 + qs - 64 + 32 - __clz(row.n)) << 23);
         it.rem = low != 0 ? it.scale * (1.f - ldexpf((float)low, -qs)) : 0.f;

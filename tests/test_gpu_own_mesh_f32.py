@@ -106,3 +106,46 @@ def test_values_that_are_not_finite(value, order, limiter):
     assert np.isfinite(got[np.isfinite(nan) & np.isfinite(ref)]).all()
     fine = np.isfinite(got) & np.isfinite(ref)
     np.testing.assert_allclose(got[fine], ref[fine], rtol=1e-5)
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-24, 1.0, 1e30])
+@pytest.mark.parametrize("length", [1e-9, 1.0, 1e13])
+@pytest.mark.parametrize("order", [2, 3])
+def test_magnitudes(order, length, scale):
+    """Values and lengths far from 1: the step is linear in the values and does not depend
+    on the unit of length (relative L1 against the FP64 oracle <= 1e-5)."""
+    n = 777
+    x = wl.random_nodes(n, seed=3) * length
+    rng = np.random.default_rng(5)
+    dx = np.diff(x)
+    q = ((1.0 + rng.random(n)) * scale).astype(np.float32).astype(np.float64)
+    dv = ((rng.random(n) - 0.5) * 1.6 * dx.min() / 0.1).astype(np.float32).astype(np.float64)
+    s = 0.3217 * length
+    plan = _plan(x, order=order)
+    got = _step(plan, q, s, dv=dv)
+    ref = oracle.step(x, q, oracle.shift_from_velocity(s / 0.1, 0.1), order, True, dv, 0.1,
+                      ram.VANLEER, 1)
+    assert plan.check_errors() == 0
+    assert np.sum(np.abs(got - ref) / scale * dx) <= 1e-5 * np.sum(np.abs(ref) / scale * dx)
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("order", [2, 3])
+def test_not_finite_with_a_residual(value, order):
+    """Cells farther than the stencils of the shift and one van Leer sub-step (7 cells on
+    each side) are as without the value, bit for bit."""
+    n = 1533
+    x = wl.random_nodes(n, seed=n + 5)
+    rng = np.random.default_rng(4)
+    q = 1.0 + rng.random(n)
+    dv = (rng.random(n) - 0.5) * 0.6 * np.diff(x).min() / 0.1
+    plan = _plan(x, order=order)
+    s = 0.2 * (x[-1] - x[0])
+    good = _step(plan, q, s, dv=dv)
+    bad = _step(plan, np.where(np.arange(n) == 700, value, q), s, dv=dv)
+    lo = np.searchsorted(x, x[700] + s) - 1
+    hi = np.searchsorted(x, x[701] + s)
+    assert not np.isfinite(bad[lo:hi]).all()
+    far = np.ones(n, dtype=bool)
+    far[lo - 7:hi + 7] = False
+    np.testing.assert_array_equal(bad[far], good[far])
