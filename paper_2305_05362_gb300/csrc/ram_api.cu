@@ -73,7 +73,7 @@ StepArgs base_args(const Plan *p, const void *q_in, void *q_out)
 // warp-segment kernels.
 bool rows_form_params(const Plan &p, ram_dtype dt, const StepArgs &a)
 {
-    if (dt != RAM_F32) return p.nseg_rows == p.n_rows;
+    if (dt != RAM_F32) return p.nseg_rows[1] == p.n_rows;
     size_t seg = 0;
     if (p.n_uniform_rows > 0) {
         if (p.uniform_kernel[0] != 1 || p.seg_variant != 2) return false;
@@ -81,7 +81,7 @@ bool rows_form_params(const Plan &p, ram_dtype dt, const StepArgs &a)
             if ((uintptr_t)ptr % 16) return false;
         for (int o = 2; o <= 4; ++o) seg += p.rows_seg_h[0][o].size();
     }
-    return seg + (size_t)(p.nu_kernel == 1 ? p.nseg_rows : 0) == (size_t)p.n_rows;
+    return seg + (size_t)(p.nu_kernel == 1 ? p.nseg_rows[0] : 0) == (size_t)p.n_rows;
 }
 
 ram_status run(const Plan *p, ram_dtype dt, const StepArgs &a0, void *stream)

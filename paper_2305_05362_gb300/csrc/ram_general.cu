@@ -648,9 +648,10 @@ struct GenList {
 
 GenList gen_list(const Plan &p, int order, bool f32)
 {
+    const int d = f32 ? 0 : 1;
     if (!f32 || p.nu_kernel == 1)
-        return {p.tiles_general32[order], (int)p.tiles_general32_h[order].size(),
-                p.gen32_whole[order], p.gen32_wcap[order], p.gen32_qcap[order]};
+        return {p.tiles_nuleft[d][order], (int)p.tiles_nuleft_h[d][order].size(),
+                p.nuleft_whole[d][order], p.nuleft_wcap[d][order], p.nuleft_qcap[d][order]};
     return {p.tiles_general[order], (int)p.tiles_general_h[order].size(), p.gen_whole[order],
             p.gen_wcap[order], p.gen_qcap[order]};
 }

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "ram.h"
+#include "ram_segments.h"
 
 namespace ram {
 
@@ -30,8 +31,9 @@ struct RowInfo {
     int32_t order;        // 2, 3, 4
     int32_t uniform;      // 1: equal widths, O(1) edge index
     int32_t bucket_bits;  // log2 of the row's bucket count
-    int32_t qshift;       // FP32 warp-segment kernel: positions are kept as 32-bit values
+    int16_t qshift;       // FP32 warp-segment kernel: positions are kept as 32-bit values
                           // (modulo 2^32) in units of 2^qshift
+    int16_t half;         // FP64 warp-segment kernel: positions in units of 2^-63, not 2^-64
     int32_t density;      // index of the row's mesh-density function, -1: none
     double period;        // L
     double cells_per_length;  // N / L
@@ -67,13 +69,16 @@ struct Tile {
 constexpr int kGenHalo = 2 * RAM_MAX_NSUB;
 constexpr int kGenHR = 2;
 
-// FP32 rows with their own mesh: the warp-segment kernel (ram_nseg.cu).  A warp
-// stages a window of kNsegWin source cells and takes segments of at most
-// kNsegMost output cells, residual halo included; a CTA of kNsegWarps warps takes
-// up to kNsegItems of them.
-constexpr int kNsegWin = 160;
-constexpr int kNsegHR = 2;          // reconstruction halo, cells per side
-constexpr int kNsegMost = kNsegWin - 8;
+// Work item of the warp-segment kernels of rows with their own mesh: one segment.
+struct NsegItem {
+    int32_t row;
+    int32_t start;
+    int32_t count;        // output cells
+    int16_t most;         // most cells of a segment with its halo (NsegFit)
+    int16_t window;       // source cells of a window that edges may lie in
+};
+
+// The FP32 one (ram_nseg.cu): a CTA of kNsegWarps warps takes up to kNsegItems items.
 constexpr int kNsegWarps = 4;
 constexpr int kNsegItems = 48;
 constexpr int kNsegCtas = 6;        // resident CTAs per SM
@@ -149,12 +154,12 @@ struct Plan {
     int32_t gen_whole[5] = {0};
     int32_t gen_wcap[5][2] = {{0}};  // [order][class]
     int32_t gen_qcap[5][2] = {{0}};
-    // the tiles of the rows the warp-segment kernels do not take (the same layout as
-    // above)
-    std::vector<Tile> tiles_general32_h[5];
-    int32_t gen32_whole[5] = {0};
-    int32_t gen32_wcap[5][2] = {{0}};
-    int32_t gen32_qcap[5][2] = {{0}};
+    // by dtype (FP32, FP64), the tiles of the rows its warp-segment kernel does not take
+    // (the same layout as above)
+    std::vector<Tile> tiles_nuleft_h[2][5];
+    int32_t nuleft_whole[2][5] = {{0}};
+    int32_t nuleft_wcap[2][5][2] = {{{0}}};
+    int32_t nuleft_qcap[2][5][2] = {{{0}}};
     // adjoint of rows with their own mesh: tiles of at most adj_nu_tcap cells per
     // order, and (flag RAM_ADJOINT) scratch for the shifted field and the residual's
     // cotangent, n_cells values each of the plan's widest dtype
@@ -169,11 +174,11 @@ struct Plan {
     // corrected averages and the remapped ones, n_cells values each (FP64 size)
     int32_t a4 = 0;
     void *a4_scratch = nullptr;
-    std::vector<Tile> tiles_nseg_h;
-    int32_t nseg_rows = 0;
+    // by dtype: the warp-segment kernel's work items, its rows and what it takes of each
+    std::vector<NsegItem> items_nseg_h[2];
+    int32_t nseg_rows[2] = {0, 0};
+    std::vector<NsegFit> nseg_fit_h[2];
     int32_t nu_kernel = 1;         // FP32 rows with their own mesh: 1 = warp-segment kernel
-    std::vector<int32_t> nseg_cells_h;  // per row: most cells of a segment with its halo, 0:
-                                        // the row does not take the warp-segment kernel
     // uniform rows taken by the persistent whole-row kernel, per dtype and order, and
     // the tiles of the remaining uniform rows
     std::vector<int32_t> rows_fit_h[2][5];
@@ -201,8 +206,8 @@ struct Plan {
     RowInfo *rows = nullptr;
     Tile *tiles_uniform[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     Tile *tiles_general[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-    Tile *tiles_general32[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-    Tile *tiles_nseg = nullptr;
+    Tile *tiles_nuleft[2][5] = {{nullptr}};
+    NsegItem *items_nseg[2] = {nullptr, nullptr};
     int32_t *rows_fit[2][5] = {{nullptr}};
     RowPos *rows_fit_pos[2][5] = {{nullptr}};
     Tile *tiles_rest[2][5] = {{nullptr}};

@@ -222,7 +222,8 @@ struct Item {
     int64_t cell_off, mesh_off;
     uint64_t S;                // the row's shift, fraction of the period in units of 2^-64
     int32_t row, n, start, count;
-    int32_t most;              // most cells of a segment with its halo
+    int16_t most;              // most cells of a segment with its halo
+    int16_t window;            // cells of a window that edges may lie in
     int32_t order;
     int32_t p;                 // source cell of the first edge (halo included)
     int32_t nsub;
@@ -590,7 +591,7 @@ __device__ __forceinline__ void nseg_segment(const SegCtx &g, uint32_t *w32, int
 
 template <bool LIM, bool RESID>
 __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
-    k_nseg(StepArgs a, const Tile *items, int n_items)
+    k_nseg(StepArgs a, const NsegItem *items, int n_items)
 {
     extern __shared__ __align__(16) uint32_t smem_w[];
     __shared__ Item s_item[kNsegItems];
@@ -605,7 +606,7 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
     // ---- one thread per item: the row's shift (S0, FP64) and the first source cell
     // (plan data is read before the wait: the previous kernel in the stream may
     // still be writing q and the phase) ----
-    Tile t{};
+    NsegItem t{};
     RowInfo row{};
     if (tid < n_it) {
         t = items[first + tid];
@@ -633,7 +634,8 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
         it.n = row.n;
         it.start = t.start;
         it.count = t.count;
-        it.most = t.window;
+        it.most = t.most;
+        it.window = t.window;
         it.order = row.order;
         it.p = locate_cell(X, row.n, a.buckets + row.bucket_off, row.bucket_bits, a.density,
                            row.density, xe - S);
@@ -716,7 +718,7 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
         g.N = it.n;
         g.H = RESID ? it.nsub * R : 0;
         g.lane = lane;
-        g.hi = kHR + min(kWin - 2 * kHR, 2 * g.N - 1);
+        g.hi = kHR + min(it.window, 2 * g.N - 1);
         g.vl = R == 2;
         g.scale = it.scale;
         g.err = a.err;
@@ -730,11 +732,11 @@ __global__ void __launch_bounds__(kNsegWarps * 32, kNsegCtas)
 
 cudaError_t launch_nseg(const Plan &p, const StepArgs &a, cudaStream_t s)
 {
-    const int n = (int)p.tiles_nseg_h.size();
+    const int n = (int)p.items_nseg_h[0].size();
     if (n == 0) return cudaSuccess;
     const bool resid = a.mode != MODE_SHIFT && a.dv != nullptr;
     const size_t smem = (size_t)kNsegWarps * (resid ? kWordsResid : kWords) * 4;
-    void (*kern)(StepArgs, const Tile *, int) =
+    void (*kern)(StepArgs, const NsegItem *, int) =
         p.limiter ? (resid ? k_nseg<true, true> : k_nseg<true, false>)
                   : (resid ? k_nseg<false, true> : k_nseg<false, false>);
     // one wave of CTAs with near-equal shares of the items (few items: one each, over
@@ -743,7 +745,7 @@ cudaError_t launch_nseg(const Plan &p, const StepArgs &a, cudaStream_t s)
     const int64_t waves = ((int64_t)n + (int64_t)wave * kNsegItems - 1) / ((int64_t)wave * kNsegItems);
     const int64_t grid = std::min<int64_t>(n, waves * wave);
     return launch_pdl(kern, dim3((unsigned)grid), dim3(kNsegWarps * 32), smem, s, a,
-                      static_cast<const Tile *>(p.tiles_nseg), n);
+                      static_cast<const NsegItem *>(p.items_nseg[0]), n);
 }
 
 }  // namespace ram

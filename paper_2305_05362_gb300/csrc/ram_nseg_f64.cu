@@ -203,7 +203,8 @@ struct Item {
     double cf;             // sub-step length in the widths' units
     double dscale;         // position units to the widths' units
     int32_t wexp;          // these are widths times 2^wexp: a mean width is in (1/2, 1]
-    int32_t row, n, start, count, most, order;
+    int32_t row, n, start, count, order;
+    int16_t most, window;
     int32_t half;          // 1: positions in units of 2^-63 of the period
     int32_t p;             // source cell of the first edge (halo included)
     int32_t nsub;
@@ -522,7 +523,7 @@ __device__ __forceinline__ void segment(const Seg &g, uint64_t *w64, int i0, int
 
 template <bool LIM, bool RESID>
 __global__ void __launch_bounds__(kWarps * 32, kCtas)
-    k_nseg_f64(StepArgs a, const Tile *items, int n_items)
+    k_nseg_f64(StepArgs a, const NsegItem *items, int n_items)
 {
     extern __shared__ __align__(16) uint64_t smem_d[];
     __shared__ Item s_item[kItems];
@@ -535,7 +536,7 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas)
     const int R = a.scheme == RAM_VANLEER ? 2 : 1;
 
     // one thread per item: the row's shift (S0) and the first source cell
-    Tile t{};
+    NsegItem t{};
     RowInfo row{};
     if (tid < n_it) {
         t = items[first + tid];
@@ -560,13 +561,14 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas)
         it.S = P.sfix;
         it.wexp = ((__double2hiint(row.cells_per_length) >> 20) & 0x7ff) - 1023;
         it.cf = P.cf * scale_pow2(1.0, it.wexp);
-        it.half = row.qshift > 32;
+        it.half = row.half;
         it.dscale = scale_pow2(row.period, it.wexp) * (it.half ? 0x1p-63 : 0x1p-64);
         it.row = t.row;
         it.n = row.n;
         it.start = t.start;
         it.count = t.count;
-        it.most = t.window;
+        it.most = t.most;
+        it.window = t.window;
         it.order = row.order;
         it.p = locate_cell(X, row.n, a.buckets + row.bucket_off, row.bucket_bits, a.density,
                            row.density, xe - P.sfix);
@@ -635,7 +637,7 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas)
         g.nsub = it.nsub;
         g.H = RESID ? it.nsub * R : 0;
         g.lane = lane;
-        g.hi = kHR + min(kWin - 2 * kHR, 2 * g.N - 1);
+        g.hi = kHR + min(it.window, 2 * g.N - 1);
         g.half = it.half;
         g.order = it.order;
         g.vl = R == 2;
@@ -665,19 +667,19 @@ cudaError_t launch_t(const Plan &p, const StepArgs &a, cudaStream_t s)
     }
     // one wave of CTAs with near-equal shares of the items, whole waves more when a
     // share would not fit the CTA's table
-    const int n = (int)p.tiles_nseg_h.size();
+    const int n = (int)p.items_nseg_h[1].size();
     const int wave = p.sm_count * kCtas;
     const int64_t waves = ((int64_t)n + (int64_t)wave * kItems - 1) / ((int64_t)wave * kItems);
     const int64_t grid = std::min<int64_t>(n, waves * wave);
     return launch_pdl(k_nseg_f64<LIM, RESID>, dim3((unsigned)grid), dim3(kWarps * 32), smem, s, a,
-                      static_cast<const Tile *>(p.tiles_nseg), n);
+                      static_cast<const NsegItem *>(p.items_nseg[1]), n);
 }
 
 }  // namespace
 
 cudaError_t launch_nseg_f64(const Plan &p, const StepArgs &a, cudaStream_t s)
 {
-    if (p.tiles_nseg_h.empty()) return cudaSuccess;
+    if (p.items_nseg_h[1].empty()) return cudaSuccess;
     const bool resid = a.mode != MODE_SHIFT && a.dv != nullptr;
     if (p.limiter)
         return resid ? launch_t<true, true>(p, a, s) : launch_t<true, false>(p, a, s);

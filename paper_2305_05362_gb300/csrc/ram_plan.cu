@@ -74,8 +74,10 @@ cudaError_t upload(T **dst, const T *src, size_t count)
 
 void free_lists(Plan &p)
 {
-    cudaFree(p.tiles_nseg);
-    p.tiles_nseg = nullptr;
+    for (int d = 0; d < 2; ++d) {
+        cudaFree(p.items_nseg[d]);
+        p.items_nseg[d] = nullptr;
+    }
     for (int o = 0; o < 5; ++o) {
         cudaFree(p.tiles_adj_nu[o]);
         p.tiles_adj_nu[o] = nullptr;
@@ -83,9 +85,10 @@ void free_lists(Plan &p)
     for (int o = 0; o < 5; ++o) {
         cudaFree(p.tiles_uniform[o]);
         cudaFree(p.tiles_general[o]);
-        cudaFree(p.tiles_general32[o]);
-        p.tiles_uniform[o] = p.tiles_general[o] = p.tiles_general32[o] = nullptr;
+        p.tiles_uniform[o] = p.tiles_general[o] = nullptr;
         for (int d = 0; d < 2; ++d) {
+            cudaFree(p.tiles_nuleft[d][o]);
+            p.tiles_nuleft[d][o] = nullptr;
             cudaFree(p.rows_fit[d][o]);
             cudaFree(p.rows_fit_pos[d][o]);
             p.rows_fit_pos[d][o] = nullptr;
@@ -133,84 +136,6 @@ std::vector<double> doubled_widths(const double *x, int n)
     std::vector<double> w2(2 * (size_t)n);
     for (int i = 0; i < n; ++i) w2[i] = w2[i + n] = x[i + 1] - x[i];
     return w2;
-}
-
-// What the FP32 warp-segment kernel takes of a row: the most cells of a segment
-// with its residual halo (0: the row is left to the tiled kernels), and the units
-// 2^qs of its 32-bit positions.  x: nodes; w: widths.
-//
-// The positions of a window and of the edges over it span less than 2^32 units; rows
-// not much longer than that take half the period's units, so that two turns fit.
-// Every cell keeps at least 2^20 units, and one output cell lies over fewer source
-// cells than a window holds (both from sums over whole rows of the widths).
-//
-// A segment whose source cells do not fit one window costs another window, so the
-// length is the one with the least expected cost per output cell, windows over
-// output cells, on 64 sampled placements (against the longest whose sampled placements
-// all fit one window: 49.9 and 51.0 us on the 512-row batch of widths within [1/2, 2] x
-// mean, 27.7 and 44.1 for the split step of 510 rings of 1533 cells on the bump mesh).
-int nseg_cells(const double *x, const double *w, int n, int &qs)
-{
-    qs = 0;
-    if (n < kNsegMinCells) return 0;
-    const int room = kNsegWin - 2 * kNsegHR;
-    const double L = x[n] - x[0];
-    if (!(L > 1e-250 && L < 1e250)) return 0;  // widths are scaled by their exponents
-    double w_min = w[0], w_max = w[0], reach = 2.0 * L;
-    for (int i = 1; i < n; ++i) {
-        w_min = std::min(w_min, w[i]);
-        w_max = std::max(w_max, w[i]);
-    }
-    const int span = kNsegWin + 2;
-    if (n > span) {
-        double len = 0.0;
-        for (int st = 0; st < n; ++st)
-            len = std::max(len, st + span <= n ? x[st + span] - x[st]
-                                               : x[st + span - n] - x[st] + L);
-        reach = len + w_max;
-    }
-    const double two64 = 18446744073709551616.0;
-    if (reach > 0.999 * L)
-        qs = 33;
-    else
-        qs = std::max(0, (int)std::ceil(std::log2(reach / L * two64 * 1.000001)) - 32);
-    if (std::ldexp(w_min / L * two64, -qs) < 1048576.0) return 0;
-    if (w_max > w_min * (room - 8)) {
-        // the most cells an interval as long as the widest cell can touch
-        int e = 0;
-        double len = 0.0;  // of cells st .. e - 1 (cyclic)
-        for (int st = 0; st < n; ++st) {
-            while (e < st + n && len + w[e % n] < w_max) len += w[e++ % n];
-            if (e - st + 2 > room - 8) return 0;
-            if (e > st)
-                len -= w[st];
-            else
-                e = st + 1;
-        }
-    }
-    int best = 0;
-    double cost = 1e300;
-    for (int ne = kNsegMost; ne >= 64; ne -= 8) {
-        const int c = std::min(ne, n - 1);
-        double windows = 0.0;
-        for (int k = 0; k < 64; ++k) {
-            const int i = (int)((2654435761ull * (2 * k + 1)) % (uint64_t)n);
-            const int j = (int)((40503ull * 65537ull * (2 * k + 1) + n / 3) % (uint64_t)n);
-            double len = (i + c <= n ? x[i + c] - x[i] : x[i + c - n] - x[i] + L) + x[j];
-            int turn = 0;
-            if (len > x[n]) {
-                len -= L;
-                turn = n;
-            }
-            const int e = (int)(std::upper_bound(x, x + n + 1, len) - x) + turn;
-            windows += std::max(1, (e - j + room - 2) / (room - 1));
-        }
-        if (windows / (c - 4) < cost) {
-            cost = windows / (c - 4);
-            best = c;
-        }
-    }
-    return best;
 }
 
 // The general kernels' per-order launch shapes of a tile list: whole-row tiles
@@ -262,14 +187,16 @@ int default_seg_warps(const Plan &p)
 ram_status build_tiles(Plan &p)
 {
     free_lists(p);
-    p.tiles_nseg_h.clear();
-    p.nseg_rows = 0;
+    for (int d = 0; d < 2; ++d) {
+        p.items_nseg_h[d].clear();
+        p.nseg_rows[d] = 0;
+    }
     for (int o = 0; o < 5; ++o) p.tiles_adj_nu_h[o].clear();
     for (int o = 0; o < 5; ++o) {
         p.tiles_uniform_h[o].clear();
         p.tiles_general_h[o].clear();
-        p.tiles_general32_h[o].clear();
         for (int d = 0; d < 2; ++d) {
+            p.tiles_nuleft_h[d][o].clear();
             p.rows_fit_h[d][o].clear();
             p.rows_fit_pos_h[d][o].clear();
             p.tiles_rest_h[d][o].clear();
@@ -342,23 +269,27 @@ ram_status build_tiles(Plan &p)
         // the adjoint's tiles: plain runs of at most adj_nu_tcap cells
         for (int a = 0; a < n; a += p.adj_nu_tcap)
             p.tiles_adj_nu_h[ri.order].push_back(Tile{r, a, std::min(p.adj_nu_tcap, n - a), 0});
-        // FP32: the warp-segment kernel's items, near-equal segments that leave room
-        // for the halo of one van Leer sub-step (wider halos are cut in the kernel)
-        const bool nseg = p.nseg_cells_h[r] > 0;
-        if (nseg) {
-            ++p.nseg_rows;
-            const int most = p.nseg_cells_h[r];
-            const int64_t ns = (n + std::max(1, most - 4) - 1) / std::max(1, most - 4);
+        // the warp-segment kernels' items, near-equal segments that leave room for the halo
+        // of one van Leer sub-step (wider halos are cut in the kernel)
+        for (int d = 0; d < 2; ++d) {
+            const NsegFit &f = p.nseg_fit_h[d][r];
+            if (f.cells == 0) continue;
+            ++p.nseg_rows[d];
+            const int64_t ns = (n + std::max(1, f.cells - 4) - 1) / std::max(1, f.cells - 4);
             for (int64_t k = 0; k < ns; ++k) {
                 const int a = (int)(n * k / ns), b = (int)(n * (k + 1) / ns);
-                p.tiles_nseg_h.push_back(Tile{r, a, b - a, most});
+                p.items_nseg_h[d].push_back(
+                    NsegItem{r, a, b - a, (int16_t)f.cells, (int16_t)f.window});
             }
         }
-        std::vector<Tile> &g32 = p.tiles_general32_h[ri.order];
+        auto add_general = [&](const Tile &t) {
+            p.tiles_general_h[ri.order].push_back(t);
+            for (int d = 0; d < 2; ++d)
+                if (p.nseg_fit_h[d][r].cells == 0) p.tiles_nuleft_h[d][ri.order].push_back(t);
+        };
         // non-uniform row: one cyclic tile for short rows, else windowed tiles
         if (n <= 2 * tg + 4 * halo_res) {
-            p.tiles_general_h[ri.order].push_back(Tile{r, 0, n, 0});
-            if (!nseg) g32.push_back(Tile{r, 0, n, 0});
+            add_general(Tile{r, 0, n, 0});
             continue;
         }
         const int nt = (n + tg - 1) / tg;
@@ -395,18 +326,19 @@ ram_status build_tiles(Plan &p)
         for (int t = 0; t < nt; ++t) {
             const int a = (int)((int64_t)n * t / nt);
             const int b = (int)((int64_t)n * (t + 1) / nt);
-            p.tiles_general_h[ri.order].push_back(Tile{r, a, b - a, window});
-            if (!nseg) g32.push_back(Tile{r, a, b - a, window});
+            add_general(Tile{r, a, b - a, window});
         }
     }
-    // tiles of one reconstruction order next to each other: CTAs that run at the
+    // items of one reconstruction order next to each other: CTAs that run at the
     // same time mostly run the same code
-    std::stable_sort(p.tiles_nseg_h.begin(), p.tiles_nseg_h.end(),
-                     [&p](const Tile &a, const Tile &b) {
-                         return p.rows_h[a.row].order < p.rows_h[b.row].order;
-                     });
-    if (upload(&p.tiles_nseg, p.tiles_nseg_h.data(), p.tiles_nseg_h.size()) != cudaSuccess)
-        return RAM_ERR_NOMEM;
+    for (int d = 0; d < 2; ++d) {
+        std::vector<NsegItem> &items = p.items_nseg_h[d];
+        std::stable_sort(items.begin(), items.end(), [&p](const NsegItem &a, const NsegItem &b) {
+            return p.rows_h[a.row].order < p.rows_h[b.row].order;
+        });
+        if (upload(&p.items_nseg[d], items.data(), items.size()) != cudaSuccess)
+            return RAM_ERR_NOMEM;
+    }
     for (int o = 2; o <= 4; ++o)
         if (upload(&p.tiles_adj_nu[o], p.tiles_adj_nu_h[o].data(), p.tiles_adj_nu_h[o].size()) !=
             cudaSuccess)
@@ -415,11 +347,13 @@ ram_status build_tiles(Plan &p)
         // the general kernel runs whole-row tiles (window 0) and windowed tiles as
         // two launches, each with the shared memory its own largest tile needs
         general_caps(p, p.tiles_general_h[o], p.gen_whole[o], p.gen_wcap[o], p.gen_qcap[o]);
-        general_caps(p, p.tiles_general32_h[o], p.gen32_whole[o], p.gen32_wcap[o],
-                     p.gen32_qcap[o]);
-        if (upload(&p.tiles_general32[o], p.tiles_general32_h[o].data(),
-                   p.tiles_general32_h[o].size()) != cudaSuccess)
-            return RAM_ERR_NOMEM;
+        for (int d = 0; d < 2; ++d) {
+            general_caps(p, p.tiles_nuleft_h[d][o], p.nuleft_whole[d][o], p.nuleft_wcap[d][o],
+                         p.nuleft_qcap[d][o]);
+            if (upload(&p.tiles_nuleft[d][o], p.tiles_nuleft_h[d][o].data(),
+                       p.tiles_nuleft_h[d][o].size()) != cudaSuccess)
+                return RAM_ERR_NOMEM;
+        }
         if (upload(&p.tiles_uniform[o], p.tiles_uniform_h[o].data(),
                    p.tiles_uniform_h[o].size()) != cudaSuccess)
             return RAM_ERR_NOMEM;
@@ -515,13 +449,13 @@ extern "C" ram_status ram_plan_mesh(const ram_mesh_desc *desc, int device, ram_p
     for (int r = 0; r < nr; ++r)
         limited4 |= p->limiter && (desc->order ? desc->order[r] : desc->default_order) == 4;
     p->rows_h.resize(nr);
-    p->nseg_cells_h.assign(nr, 0);
+    for (int d = 0; d < 2; ++d) p->nseg_fit_h[d].assign(nr, NsegFit());
     for (int r = 0; r < nr && st == RAM_OK; ++r) {
         const int n = (int)(ro[r + 1] - ro[r]);
         const double *x = shared ? p->nodes_h.data() : p->nodes_h.data() + ro[r] + r;
         RowInfo &ri = p->rows_h[r];
         ri.density = -1;
-        ri.qshift = 0;
+        ri.qshift = ri.half = 0;
         ri.cell_off = ro[r];
         ri.n = n;
         ri.order = desc->order ? desc->order[r] : desc->default_order;
@@ -535,7 +469,8 @@ extern "C" ram_status ram_plan_mesh(const ram_mesh_desc *desc, int device, ram_p
             ri.bucket_off = p->rows_h[0].bucket_off;
             ri.bucket_bits = p->rows_h[0].bucket_bits;
             ri.qshift = p->rows_h[0].qshift;
-            p->nseg_cells_h[r] = p->nseg_cells_h[0];
+            ri.half = p->rows_h[0].half;
+            for (int d = 0; d < 2; ++d) p->nseg_fit_h[d][r] = p->nseg_fit_h[d][0];
             continue;
         }
         st = check_nodes(x, n);
@@ -568,10 +503,11 @@ extern "C" ram_status ram_plan_mesh(const ram_mesh_desc *desc, int device, ram_p
         }
         x32.resize(base + n);
         if (!ri.uniform) {
-            int qs = 0;
-            p->nseg_cells_h[r] = nseg_cells(x, dx64.data() + base, n, qs);
-            ri.qshift = qs;
-            for (int i = 0; i < n; ++i) x32[base + i] = (uint32_t)(xfix[base + i] >> qs);
+            for (int d = 0; d < 2; ++d)
+                p->nseg_fit_h[d][r] = nseg_fit(x, dx64.data() + base, n, kNsegMinCells, d == 0);
+            ri.qshift = (int16_t)p->nseg_fit_h[0][r].units;
+            ri.half = (int16_t)p->nseg_fit_h[1][r].units;
+            for (int i = 0; i < n; ++i) x32[base + i] = (uint32_t)(xfix[base + i] >> ri.qshift);
         }
         int bits = 1;
         while ((1LL << bits) < 2LL * n && bits < 40) ++bits;
@@ -656,7 +592,7 @@ extern "C" ram_status ram_plan_query(ram_plan plan, ram_plan_info *info)
     info->tile_cells = p->tile_cells;
     info->threads = p->threads;
     info->device = p->device;
-    info->n_nseg_rows = p->nseg_rows;
+    info->n_nseg_rows = p->nseg_rows[0];
     int nd = 0;
     for (const RowInfo &ri : p->rows_h) nd += ri.density >= 0 ? 1 : 0;
     info->n_density_rows = nd;

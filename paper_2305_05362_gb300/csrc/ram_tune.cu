@@ -189,7 +189,7 @@ extern "C" ram_status ram_plan_autotune(ram_plan plan, ram_dtype dtype, const vo
     for (int o = 2; o <= 4; ++o) {
         any_tiles |= p->uniform_kernel[d] == 0 ? !p->tiles_rest_h[d][o].empty()
                                                : !p->tiles_rest_seg_h[d][o].empty();
-        any_tiles |= d == 1 || p->nu_kernel == 1 ? !p->tiles_general32_h[o].empty()
+        any_tiles |= d == 1 || p->nu_kernel == 1 ? !p->tiles_nuleft_h[d][o].empty()
                                                  : !p->tiles_general_h[o].empty();
     }
     if (any_tiles && st == RAM_OK) {
@@ -216,7 +216,7 @@ extern "C" ram_status ram_plan_autotune(ram_plan plan, ram_dtype dtype, const vo
         ram_status r = ram_plan_set_tiling(plan, best_tc, best_th);
         if (st == RAM_OK) st = r;
     }
-    if (d == 0 && p->nseg_rows > 0 && st == RAM_OK) {
+    if (d == 0 && p->nseg_rows[0] > 0 && st == RAM_OK) {
         // FP32 rows with their own mesh: the warp-segment kernel or the per-order ones
         int best_nu = p->nu_kernel;
         float best = 3.4e38f;
