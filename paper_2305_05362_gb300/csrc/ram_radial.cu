@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(kCols) k_radial(int nr, int N, const T *q, T *
             if (k < nr) {
                 const double r1 = rf[k + 1];
                 g.w = (T)(r1 - r0);
-                g.ka = (T)dt / (T)(0.5 * (r1 - r0) * (r1 + r0));
+                g.ka = (T)(dt / (0.5 * (r1 - r0) * (r1 + r0)));
                 if (k > 0) g.spacing = (T)(0.5 * (r1 - rf[k - 1]));
             }
             ring[threadIdx.x] = g;
