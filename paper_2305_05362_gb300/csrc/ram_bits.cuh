@@ -19,6 +19,11 @@ __device__ __forceinline__ unsigned long long mag_up(unsigned long long m, int k
 {
     return (m >> 52) == 0 ? 0ull : m + ((unsigned long long)k << 52);
 }
+// |x| > |y|, false where x is NaN
+__device__ __forceinline__ bool mag_above(double x, double y)
+{
+    return mag(x) > mag(y) && mag(x) <= 0x7ff0000000000000ull;
+}
 __device__ __forceinline__ unsigned long long mag_min(unsigned long long a, unsigned long long b)
 {
     return a < b ? a : b;

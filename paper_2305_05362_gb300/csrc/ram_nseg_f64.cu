@@ -506,7 +506,7 @@ __device__ __forceinline__ void segment(const Seg &g, uint64_t *w64, int i0, int
 #pragma unroll
         for (int i = 0; i < kV; ++i)
             bad |= b + i >= R && b + i <= ne - R &&
-                   mag(c[i]) > mag(__double_as_longlong(c[i]) > 0 ? (i ? h[i - 1] : hm) : h[i]);
+                   mag_above(c[i], __double_as_longlong(c[i]) > 0 ? (i ? h[i - 1] : hm) : h[i]);
         if (__any_sync(kFull, bad) && lane == 0) atomicOr(g.err, ERR_CFL);
         if (odd)
             residual<false>(cur, c, h, rh, g.nsub, g.vl);

@@ -774,7 +774,7 @@ __device__ __forceinline__ void seg_f64(const StepArgs &a, const RowParams<doubl
 #pragma unroll
         for (int i = 0; i < V; ++i) {
             c[i] *= P.cf;
-            bad |= mag(c[i]) > 0x3ff0000000000000ull;  // |c| > 1
+            bad |= mag_above(c[i], 1.0);
             if (VL) wc[i] = (__double_as_longlong(c[i]) > 0 ? 1.0 : -1.0) - c[i];
         }
         if (bad) atomicOr(a.err, ERR_CFL);
