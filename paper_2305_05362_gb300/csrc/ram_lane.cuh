@@ -186,8 +186,10 @@ template <typename T, int M> __device__ __forceinline__ void a4_average(T (&q)[M
 // with D the second difference and M = 1 + D / 24, so that the recursions run on the
 // small D <Q> and their rounding with it; M^-1 / 24 = -r times the two recursions.  A
 // lane's starts with what its neighbours' bring: the next lane's alone (r^V of the one
-// beyond: below FP32 rounding for V = 8), in FP64 the next two.
-template <typename T, int V> __device__ __forceinline__ void a4_points(T (&x)[V])
+// beyond: below FP32 rounding for V = 8), in FP64 the next two.  Returns whether a value
+// is not finite: the recursions carry it through whole lanes, and the caller takes
+// a4_points_any then.
+template <typename T, int V> __device__ __forceinline__ bool a4_points(T (&x)[V])
 {
     const unsigned full = 0xffffffffu;
     const T r = (T)kA4Root;
@@ -215,6 +217,10 @@ template <typename T, int V> __device__ __forceinline__ void a4_points(T (&x)[V]
     if (sizeof(T) == 8) c = fma(rp[V - 1], __shfl_down_sync(full, t[0], 2), c);
 #pragma unroll
     for (int i = 0; i < V; ++i) x[i] = fma(r, fma(rp[V - 1 - i], c, t[i]), x[i]);
+    // t[0] holds a share of all the lane's values
+    if (sizeof(T) == 8)
+        return __any_sync(full, (__double2hiint((double)t[0]) & 0x7ff00000) == 0x7ff00000);
+    return __any_sync(full, !(fabsf((float)t[0]) < INFINITY));
 }
 
 // One residual sub-step for V cells m0..m0+V-1.  z[0..V+3] holds Q at cells
@@ -418,6 +424,43 @@ __device__ __forceinline__ void residual_group_cs(const T (&z)[V + 4], const T (
     for (int k = 0; k < V; ++k) out[k] = z[k + 2] - (F[k + 1] - F[k]);
 }
 
+// The point values of cells m0 .. m0 + V - 1 of a row of N >= 32 cells straight from its
+// input: the averages, remapped, with the inverse's weights out to 12 cells (k_a4_point in
+// ram_a4.cu), so that what is not finite reaches no farther than there.
+template <typename T, bool LIM, int V>
+__device__ __noinline__ void a4_points_any(const T *row, int N, RowParams<T> P, int m0, T *out)
+{
+    T acc[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc[v] = T(0);
+    for (int j = -12; j < V + 12; ++j) {
+        int c = (m0 + j - P.K - 4) % N;  // p - 3, p the source cell of cell m0 + j
+        c = c < 0 ? c + N : c;
+        T q[8], a[6], x[1];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            q[i] = row[c];
+            c = c + 1 < N ? c + 1 : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < 6; ++i)
+            a[i] = q[i + 1] + (q[i + 2] - T(2) * q[i + 1] + q[i]) * (T(1) / T(24));
+        if (sizeof(T) == 4)
+            remap_group<T, 3, 1>(a, P, LIM, x);
+        else
+            remap_group_cs<T, 3, 1>(a, P, LIM, x);
+        // r^|j - v| / (22 + 2 r), 0 beyond 12 cells (where it is not added: 0 times NaN)
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            const int d = j < v ? v - j : j - v;
+            double w = 1.0 / (22.0 + 2.0 * kA4Root);
+            for (int k = 0; k < d; ++k) w *= kA4Root;
+            if (d <= 12) acc[v] += (T)w * x[0];
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) out[v] = T(24) * acc[v];
+}
 
 // ---------------------------------------------------------------------------
 // Packed FP32 forms: two segments per lane, one per half of a float2.

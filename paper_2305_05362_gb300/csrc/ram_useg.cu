@@ -304,13 +304,14 @@ __device__ __forceinline__ void window_at(const float4 (&xw)[(V + 12) / 4], int 
 // vectors, in registers: the remap of the lane's V cells, the residual sub-steps with
 // shuffled neighbours, and the store of the segment's interior (whole vectors; the
 // cells past N belong to no segment).  m0: the lane's first cell; store_end: see
-// store_ends.  Shared by the register-prefetch and shared-memory-ring kernels.
+// store_ends.  Shared by the register-prefetch and shared-memory-ring kernels.  qin: the
+// row's input (A4).
 template <int ORDER, int V, bool LIM, bool VL, bool A4 = false>
 __device__ __forceinline__ void seg_compute_f32(const RowParams<float> &P, int nsub, int m0,
                                                 bool use_dv, const int (&store_end)[V / 4],
                                                 float (&q)[V + 5],
                                                 const float4 (&xv)[V / 4], float *qout,
-                                                float &cmax)
+                                                float &cmax, const float *qin = nullptr)
 {
     constexpr int VEC = 4;
     float cur[V];
@@ -319,7 +320,14 @@ __device__ __forceinline__ void seg_compute_f32(const RowParams<float> &P, int n
         remap_warp3<V>(q, P, LIM, cur);
     else
         remap_group<float, ORDER, V>(q, P, LIM, cur);
-    if constexpr (A4) a4_points(cur);
+    if constexpr (A4) {
+        if (a4_points(cur)) {
+            float x[V];
+            a4_points_any<float, LIM, V>(qin, P.n, P, m0, x);
+#pragma unroll
+            for (int k = 0; k < V; ++k) cur[k] = x[k];
+        }
+    }
     if (use_dv) {
         float v[V];
 #pragma unroll
@@ -609,7 +617,7 @@ __global__ void __launch_bounds__(256, 3)
         __syncwarp();
         issue(i + L::S);
         seg_compute_f32<ORDER, V, LIM, VL, A4>(P, nsub, seg * stride + lane_m0, use_dv, store_end, q,
-                                               xv, qout, cmax);
+                                               xv, qout, cmax, qin);
     }
     cp_async_wait<0>();
     if (cmax > 1.0f) atomicOr(a.err, ERR_CFL);
@@ -766,7 +774,14 @@ __device__ __forceinline__ void seg_f64(const StepArgs &a, const RowParams<doubl
 #pragma unroll
         for (int k = 0; k < V; ++k) cur[k] = (q[k + 2] - A[k]) + A[k + 1];
     }
-    if (A4) a4_points(cur);
+    if constexpr (A4) {
+        if (a4_points(cur)) {
+            double x[V];
+            a4_points_any<double, LIM, V>(qin, N, P, m0, x);
+#pragma unroll
+            for (int k = 0; k < V; ++k) cur[k] = x[k];
+        }
+    }
     // ---- residual sub-steps (residual_group_cs's flux, each formed once) ----
     if (has_dv) {
         double wc[V];  // the swept part's midpoint: +-1 - c
