@@ -26,6 +26,7 @@
 #include <cstdint>
 #include <vector>
 
+#include "ram_bits.cuh"
 #include "ram_device.cuh"
 
 namespace ram {
@@ -88,6 +89,21 @@ __device__ __forceinline__ int wrap_twice(int c, int N)  // c within (-2N, 2N)
     if (c >= N) c -= N;
     if (c >= N) c -= N;
     return c;
+}
+
+// Whether x is above 0 (or a NaN); whether x, not -0.0, is at least 0 and below 0 (FP64: on
+// the integer pipe)
+__device__ __forceinline__ bool above_0(float x) { return x > 0.f; }
+__device__ __forceinline__ bool above_0(double x) { return __double_as_longlong(x) > 0; }
+__device__ __forceinline__ bool upward(float x) { return x >= 0.f; }
+__device__ __forceinline__ bool downward(float x) { return x < 0.f; }
+__device__ __forceinline__ bool upward(double x)
+{
+    return (unsigned long long)__double_as_longlong(x) <= 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool downward(double x)
+{
+    return __double2hiint(x) < 0 && mag(x) <= 0x7ff0000000000000ull;
 }
 
 template <typename T> struct Vec16;
@@ -155,18 +171,20 @@ __device__ __forceinline__ void adj_segment(const StepArgs &a, const RowInfo &ro
     T g[V];
     load_cells<T, V, V>(g_out + row.cell_off, mw, lane, N, g);
     if (nsub > 0) {
-        T cp[V + 1], cm[V];  // upwind parts of the faces' Courant numbers (face i: left node)
-        {
-            T c[V];
-            load_cells<T, V, V>(static_cast<const T *>(a.dv) + row.cell_off, mw, lane, N, c);
+        // the faces' Courant numbers (face i: left node), and bit i of `up`, `down`: c[i] is
+        // at least 0, below 0 (neither for a NaN).  A cell takes nothing from a face that it
+        // is downwind of: there 0 times what is not finite would reach it
+        T c[V];
+        unsigned up = 0, down = 0;
+        load_cells<T, V, V>(static_cast<const T *>(a.dv) + row.cell_off, mw, lane, N, c);
 #pragma unroll
-            for (int i = 0; i < V; ++i) {
-                c[i] *= P.cf;
-                cp[i] = fmax(c[i], T(0));
-                cm[i] = fmin(c[i], T(0));
-            }
-            cp[V] = __shfl_down_sync(full, cp[0], 1);
+        for (int i = 0; i < V; ++i) {
+            c[i] = fma(c[i], P.cf, T(0));  // -0.0: 0.0
+            up |= upward(c[i]) ? 1u << i : 0u;
+            down |= downward(c[i]) ? 1u << i : 0u;
         }
+        const T cr = __shfl_down_sync(full, c[0], 1);
+        up |= (__shfl_down_sync(full, up, 1) & 1u) << V;
         T acc[V], q0[V];
 #pragma unroll
         for (int i = 0; i < V; ++i) acc[i] = T(0);
@@ -205,7 +223,8 @@ __device__ __forceinline__ void adj_segment(const StepArgs &a, const RowInfo &ro
                     const T zl = __shfl_up_sync(full, q[V - 1], 1);
                     T F[V + 1];
 #pragma unroll
-                    for (int i = 0; i < V; ++i) F[i] = fma(cp[i], i ? q[i - 1] : zl, cm[i] * q[i]);
+                    for (int i = 0; i < V; ++i)
+                        F[i] = c[i] * (above_0(c[i]) ? (i ? q[i - 1] : zl) : q[i]);
                     F[V] = __shfl_down_sync(full, F[0], 1);
 #pragma unroll
                     for (int i = 0; i < V; ++i) q[i] -= F[i + 1] - F[i];
@@ -214,12 +233,15 @@ __device__ __forceinline__ void adj_segment(const StepArgs &a, const RowInfo &ro
 #pragma unroll
                 for (int i = 0; i < V; ++i) {
                     // the upwind cell, the left one at c = 0
-                    const T qu = cm[i] < T(0) ? q[i] : (i ? q[i - 1] : zl);
+                    const T qu = up >> i & 1u ? (i ? q[i - 1] : zl) : q[i];
                     acc[i] = fma(qu, h[i], acc[i]);
                 }
             }
 #pragma unroll
-            for (int i = 0; i < V; ++i) g[i] = fma(cp[i + 1], h[i + 1], fma(cm[i], h[i], g[i]));
+            for (int i = 0; i < V; ++i) {
+                if (down >> i & 1u) g[i] = fma(c[i], h[i], g[i]);
+                if (up >> (i + 1) & 1u) g[i] = fma(i + 1 < V ? c[i + 1 < V ? i + 1 : 0] : cr, h[i + 1], g[i]);
+            }
         }
         if (g_dv != nullptr) {
             T *gd = g_dv + row.cell_off;
