@@ -58,8 +58,9 @@ __device__ __forceinline__ double pow2_below(double x, int sign)
 }
 
 // x y > 0, |x| > 2|y|: on the integer pipe in FP64 (x y > 0 also asks that the product
-// does not vanish and neither is NaN)
-__device__ __forceinline__ bool positive(float x, float y) { return x * y > 0.f; }
+// does not vanish and neither is NaN); in FP32 by the signs alone, as in the forward
+// kernel (the product vanishes below 1e-22)
+__device__ __forceinline__ bool positive(float x, float y) { return minxs_nan(x, y) > 0.f; }
 __device__ __forceinline__ bool positive(double x, double y)
 {
     const int hx = __double2hiint(x), hy = __double2hiint(y);
