@@ -503,10 +503,11 @@ extern "C" ram_status ram_plan_mesh(const ram_mesh_desc *desc, int device, ram_p
         }
         x32.resize(base + n);
         if (!ri.uniform) {
-            for (int d = 0; d < 2; ++d)
-                p->nseg_fit_h[d][r] = nseg_fit(x, dx64.data() + base, n, kNsegMinCells, d == 0);
-            ri.qshift = (int16_t)p->nseg_fit_h[0][r].units;
-            ri.half = (int16_t)p->nseg_fit_h[1][r].units;
+            NsegFit fit[2];
+            nseg_fit(x, dx64.data() + base, n, kNsegMinCells, fit);
+            for (int d = 0; d < 2; ++d) p->nseg_fit_h[d][r] = fit[d];
+            ri.qshift = (int16_t)fit[0].units;
+            ri.half = (int16_t)fit[1].units;
             for (int i = 0; i < n; ++i) x32[base + i] = (uint32_t)(xfix[base + i] >> ri.qshift);
         }
         int bits = 1;

@@ -21,7 +21,9 @@ extern "C" void fit(const double *x, int n, int least, int f32, int *out)
 {
     double *w = new double[n];
     for (int i = 0; i < n; ++i) w[i] = x[i + 1] - x[i];
-    const ram::NsegFit f = ram::nseg_fit(x, w, n, least, f32 != 0);
+    ram::NsegFit both[2];
+    ram::nseg_fit(x, w, n, least, both);
+    const ram::NsegFit f = both[f32 ? 0 : 1];
     delete[] w;
     out[0] = f.cells; out[1] = f.window; out[2] = f.units;
 }
