@@ -294,7 +294,9 @@ __device__ __forceinline__ void adj_segment(const StepArgs &a, const RowInfo &ro
 //
 // Bound by latency at 512 x 2048 cells, where a step's 24 bytes a cell stay in L2:
 // steps back to back, one or two sub-steps, PPM, 28.6 us with the tile passes of
-// k_adj_uniform and the parameter kernel before them, 8.7 so (FP32; FP64 103 and 63).
+// k_adj_uniform and the parameter kernel before them, 8.7 so (FP32; FP64 103 and 63;
+// with the upwind sides selected by masks, which took 9.1 to 9.2 us in FP32 timed by
+// itself, 58).
 // A segment a warp, so that few rows still fill the SMs; registers capped for six
 // CTAs an SM in FP32 (9.25 us uncapped).
 template <typename T, int ORDER>

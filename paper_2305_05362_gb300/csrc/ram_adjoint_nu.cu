@@ -461,8 +461,9 @@ cudaError_t launch_adj_nu_t(const Plan &p, const StepArgs &a, const void *g_out,
             b.n_tiles = nt;
             const RowParams<T> *pars = static_cast<const RowParams<T> *>(p.row_par);
             if (first) {
-                // the shift launches above do not wait for each other: the first
-                // reader of the scratch takes the stream's full ordering
+                // the first reader of the scratch takes the stream's full ordering (the
+                // launches above wait for each other at their end, so a programmatic
+                // launch would do)
                 k_adj_resid_nu<T><<<nt, 256, smem, s>>>(b, pars, qs, static_cast<const T *>(g_out),
                                                          gprime, static_cast<T *>(g_dv), tcap);
                 e = cudaGetLastError();

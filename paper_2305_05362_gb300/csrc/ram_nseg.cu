@@ -32,7 +32,8 @@
 // Positions are 32-bit fixed point, in units of 2^qshift of the plan's 64-bit
 // fraction of the period.  A power-of-two number of units makes the period 2^32
 // (or a multiple of it), so that differences modulo 2^32 need no case for the
-// wrap; the plan picks qshift so that a window spans less than 2^32 units and
+// wrap; the plan (nseg_fit in ram_segments.h) picks qshift, and how many of a window's
+// cells are used, so that a window spans less than 2^32 units and
 // every cell at least 2^20 (a mean cell about 2^24).  Source and output widths,
 // positions and offsets all come from the same rounded nodes, so that what the
 // rounding does is to move the mesh by 2^-24 of a mean cell: the masses stay
@@ -44,8 +45,8 @@
 // 8.8e-8 on the 512-row batch).
 //
 // Why this form: at 16 bytes a cell the step is bound by the instructions it
-// issues and by the shared-memory passes of its gathers, not by DRAM (61% of the
-// issue slots, 70% of the shared-memory data path, 24% of the measured bandwidth on
+// issues and by the shared-memory passes of its gathers, not by DRAM (60% of the
+// issue slots, 72% of the shared-memory data path, 25% of the measured bandwidth on
 // the 512-row batch).  Five cells per lane, an odd number, keep every strided access
 // of the shared arrays free of bank conflicts (16-byte ones too), pay for the search
 // once per five edges, and form the stencil's differences and reciprocals once per
@@ -56,12 +57,15 @@
 // The last quotient (Eq. 26) takes a correction step: it costs 2% (50.2 us against 49.3)
 // and keeps the error below the per-order kernels' over batches of rows (8.8e-8 against
 // 1.1e-7, relative 2-norm; 9.3e-8 without) and level with theirs on meshes graded 16:1
-// (0.77 to 1.13 times, 0.96 in the mean over 20 split steps; 0.79 to 1.19 without).
+// (0.77 to 1.13 times, 0.96 in the mean over 20 split steps; 0.79 to 1.19 without).  Over 1000
+// steps of a steady rotation on the 16:1 bump mesh the masses stay within 1e-7 and the
+// field within 8e-7 of the exact one (per-order kernels 5e-5 each, 510 cells).
 //
 // Measured against the per-order kernels (k_params with k_gwarp, or k_general with a
 // residual), us per step: 512 rows of 64 to 65536 cells (5.3 M cells), no limiter,
-// 112.6 / 50.2, with a van Leer residual 204.8 / 67.1; 1000 rows (9.5 M) limited
-// 198.6 / 90.3; one row of 4096 cells with a residual 14.3 / 7.8.  Tried (when the batch
+// 112.6 / 51.0, with a van Leer residual 204.8 / 67.6; 1000 rows (9.5 M) limited
+// 198.6 / 91.0; one row of 4096 cells with a residual 14.3 / 7.8.  Limited, 16 bytes (24 with
+// a residual) of registers a thread are spilled at the cap of 80 for six CTAs an SM.  Tried (when the batch
 // took 52.0): seven cells per lane 57.5 (512 rows), seven or five CTAs per SM instead of
 // six 52.9 and 52.9, the lane's edges by side-by-side halvings instead of the walk 54.7,
 // a loop without the two predicated steps 54.9, the next node's position kept across

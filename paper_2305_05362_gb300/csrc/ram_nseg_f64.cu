@@ -1,16 +1,19 @@
 // RAM step on FP64 rows with their own non-uniform mesh (Sec. 3 on an arbitrary
 // periodic mesh): the warp-segment form of ram_nseg.cu in double precision.
 //
-// The same work items, windows, walk and residual as the FP32 kernel, on the plan's
-// 64-bit positions (modulo 2^64, the period; rows about as long as a window or
-// shorter halve the units, so that two turns fit) and FP64 widths.  What differs is
+// The same windows, walk and residual as the FP32 kernel, on items of its own (nseg_fit in
+// ram_segments.h), the plan's 64-bit positions (modulo 2^64, the period; rows about as
+// long as a window or shorter halve the units, so that two turns fit) and FP64 widths.
+// What differs is
 // what bounds it: the FP64 pipe, which takes a warp instruction every 16 cycles of an
 // SM.  So every reconstruction is formed once per cell, its shared terms once per
 // face (neighbours by shuffles), the limiters decide on the bits, and quotients are
 // Newton steps (ram_bits.cuh): about 46 FP64 instructions per source cell and 12 per
 // edge for PPM.  The tiled kernels formed the reconstruction of the source cell at
 // every edge, three delta<Q> and two faces each time, with range-checked divides: over
-// 500 instructions a cell, the FP64 pipe 87-89% busy.
+// 500 instructions a cell, the FP64 pipe 87-89% busy.  At the cap of 168 registers for
+// three CTAs an SM the residual forms spill 316 (limited) and 188 bytes a thread, the
+// limited shift 16.
 //
 // A window that holds a value of 2^1000 or more in magnitude, an infinity or a NaN, or
 // only values below 2^-400, has its limiters decided by floating-point comparisons

@@ -487,7 +487,7 @@ struct RingLayout {
 // registers before the remap and the point values recovered after it (a4_average,
 // a4_points), with a wider halo: one launch and 12 bytes a cell, against four kernels
 // that passed the field through memory between them (512 x 4096 cells with a
-// residual, steps back to back: 46.9 and 10.3 us).
+// residual, steps back to back: 46.9 and 10.5 us).
 template <int ORDER, int V, bool LIM, bool VL, bool A4>
 __global__ void __launch_bounds__(256, 3)
     k_useg_ring(StepArgs a, const int32_t *row_ids)
@@ -966,9 +966,9 @@ cudaError_t launch_useg_f32(const Plan &p, const StepArgs &a, cudaStream_t s, in
 }  // namespace
 
 // Rows for this kernel: the plan's warp-segment list (16-byte aligned rows of at
-// least 512 cells, so that a lane's window wraps the row at most once); 8 (FP32)
-// or 4 (FP64) cells per lane.  FP32 takes the plan's variant: 0 one segment in
-// flight per warp, 1 the next segment's loads in flight in registers, 2 a ring of
+// least 512 cells, so that a lane's window wraps the row at most once); 8 cells per
+// lane.  FP64 has one form and one shape; FP32 takes the plan's warps per row CTA and
+// its variant: 0 one segment in flight per warp, 1 the next segment's loads in flight in registers, 2 a ring of
 // shared-memory stages per warp (with the shift parameters formed in the kernel).
 cudaError_t launch_useg(const Plan &p, ram_dtype dt, const StepArgs &a, cudaStream_t s,
                         int order, const int32_t *row_ids, int n_rows, int longest)
