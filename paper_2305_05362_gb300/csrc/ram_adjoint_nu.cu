@@ -96,10 +96,13 @@ __device__ __forceinline__ void overlap_moments(const StepArgs &a, const RowInfo
 #pragma unroll
     for (int k = 0; k < K; ++k) nu[k] = T(0);
     T u = divided ? gp[i] : gp[i] * rcp(DX[i] * wscale);
-    // the shifted cell [y0, y0 + wp) overlaps output cells i, i + 1, ...
+    // the shifted cell [y0, y0 + wp) overlaps output cells i, i + 1, ..., at the last the
+    // first one again (a cell that spans all the others): its right end is behind then
+    uint64_t walked = 0;
     for (int guard = 0; guard <= N; ++guard) {
         const uint64_t rr = (i + 1 < N ? X[i + 1] : 0ull) - y0;  // output cell's right end
-        if (rr >= wp) break;
+        if (rr >= wp || rr <= walked) break;
+        walked = rr;
         i = i + 1 < N ? i + 1 : 0;
         const T un = divided ? gp[i] : gp[i] * rcp(DX[i] * wscale);
         const T xi = u64f(rr, T(0)) * iw;
