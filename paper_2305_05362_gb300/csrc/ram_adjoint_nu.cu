@@ -50,6 +50,10 @@ __device__ __forceinline__ double u64f(uint64_t v, double) { return u64_to_doubl
 __device__ __forceinline__ float rcp(float x) { return rcp_approx(x); }
 __device__ __forceinline__ double rcp(double x) { return rcp_newton(x); }
 
+// x y rounded, not joined with a sum
+__device__ __forceinline__ float mul_rn(float x, float y) { return __fmul_rn(x, y); }
+__device__ __forceinline__ double mul_rn(double x, double y) { return __dmul_rn(x, y); }
+
 // 2^e (sign = 1) or 2^-e (sign = -1), e the exponent of the normal x
 __device__ __forceinline__ double pow2_below(double x, int sign)
 {
@@ -372,9 +376,10 @@ __global__ void __launch_bounds__(256)
     for (int k = ns - 1; k >= 0; --k) {
         const T *qk = st + (size_t)k * wc;
         const int lo = ns - k, hi = nc - (ns - k);  // g^(k) valid on [lo, hi)
-        // lf_j for interfaces j in [lo, hi]: g_j / dx_j - g_{j-1} / dx_{j-1}
+        // lf_j for interfaces j in [lo, hi]: g_j / dx_j - g_{j-1} / dx_{j-1}, each rounded
+        // alike on both sides of its cell, so that what the interfaces take cancels
         for (int j = lo + tid; j <= hi; j += nth)
-            lf[j] = cur[j] * rd[j] - cur[j - 1] * rd[j - 1];
+            lf[j] = mul_rn(cur[j], rd[j]) - mul_rn(cur[j - 1], rd[j - 1]);
         __syncthreads();
         if (gd)
             for (int j = ns + tid; j < ns + tn; j += nth) {
