@@ -2,8 +2,8 @@
 // periodic mesh), and the per-row mass diagnostic.
 //
 // These kernels take the rows that the warp-segment kernels (ram_nseg.cu,
-// ram_nseg_f64.cu) do not: shorter than kNsegMinCells, or graded beyond one of their
-// windows, and FP32 rows where the plan's tuning asks for them.  Steps without a
+// ram_nseg_f64.cu) do not (nseg_fit in ram_segments.h): shorter than kNsegMinCells, or
+// graded beyond one of their windows, and FP32 rows where the plan's tuning asks for them.  Steps without a
 // residual run k_gwarp (below): warps split each tile, each lane locates its own edges
 // and gathers the source stencils from the cache, with no shared memory or barriers.
 // Steps with a residual run k_general:
